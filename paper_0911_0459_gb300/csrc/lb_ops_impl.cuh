@@ -42,6 +42,25 @@ static inline int grid_for(size_t n, int threads) {
   return (int)(b > cap ? cap : (b < 1 ? 1 : b));
 }
 
+// Launch of a step kernel that may start while the previous one on the stream
+// still runs (pdl_wait in lb_device.cuh); captured into a graph, the dependency
+// becomes a programmatic edge.
+template <class Args>
+static cudaError_t launch_pdl(void (*kernel)(Args), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                              const Args& k) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, k);
+}
+
 template <int MODEL, class S, int BX>
 static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
   StepArgs<MODEL, S> k;
@@ -52,8 +71,7 @@ static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
   k.dst = to_buf<S>(a.dst, a);
   k.yc = a.yc;
   const unsigned grid = tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc);
-  step_kernel<MODEL, S, BX><<<grid, BX, 0, s>>>(k);
-  return cudaGetLastError();
+  return launch_pdl(step_kernel<MODEL, S, BX>, grid, BX, 0, s, k);
 }
 
 template <int MODEL, class S, int BX, int NS>
@@ -75,8 +93,7 @@ static cudaError_t launch_staged(const OpArgs& a, cudaStream_t s) {
   k.yc = a.yc;
   k.err = a.err;
   const unsigned grid = tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc);
-  step_tma_kernel<MODEL, S, BX, NS><<<grid, BX + 32, L::BYTES, s>>>(k);
-  return cudaGetLastError();
+  return launch_pdl(step_tma_kernel<MODEL, S, BX, NS>, grid, BX + 32, L::BYTES, s, k);
 }
 
 template <int NW, class S>

@@ -732,11 +732,13 @@ __global__ void __launch_bounds__(BX + 32, (tma_min_blocks_of<MODEL, S, BX, NS>(
   const int xb = cb * BX;
   const int y0 = band * a.yc;
   const int y1 = min(y0 + a.yc, a.G.ny);
-  if (tile_all_solid(a.G, xb, min(BX, a.G.nx - xb), y0, y1)) return;  // CTA-uniform, before any barrier
+  if (tile_all_solid(a.G, xb, min(BX, a.G.nx - xb), y0, y1)) return;  // CTA-uniform; touches no state
+  pdl_wait();
   if (warp == BX / 32) {
     if (lane != 0) return;
     unsigned issued = 0;
     if (!produce_tile<MODEL, S, BX, NS>(R, a.G, a.src, xb, y0, y1, 0u, issued)) atomicExch(a.err, 1);
+    pdl_trigger();
     drain_ring<MODEL, S, BX, NS>(R, issued);
     return;
   }
