@@ -319,6 +319,64 @@ static lb_status default_state(lb_ctx* c) {
   return upload_and_init(c, rho.data(), z.data(), z.data(), phi.data(), true);
 }
 
+// Tile of a new lattice (lb_set_tile and lb_autotune replace it): columns per CTA by
+// kernel, and as many rows per band as put the fluid tiles of the lattice on the GPU
+// in one wave of resident CTAs, up to the band at which the kernel is fastest on
+// lattices of many waves.  A small lattice with the bands of a large one leaves most
+// SMs idle (256 x 32 FP64 at 128 x 16 is four CTAs); bands of one row recompute the
+// sums of two halo rows for each row, which no longer pays once a wave is full.
+// Measured in us per step, 128 x 16 for every lattice against this rule:
+//   256 x 32 liquid-gas FP64      84.0   9.0 (64 x 1)
+//   700 x 40 FP32 planes          15.8   3.5 (128 x 1)
+//   2048 x 64 FP32 planes         27.1   7.4 (256 x 1)      FP32 blocks  13.6   5.5 (128 x 2)
+//   4096 x 128 FP32 blocks        17.6  11.2 (128 x 6)      moments      15.0  11.3 (128 x 6)
+//   16384 x 256 FP32 blocks       85.4  79.6 (128 x 8)      moments      50.5  48.2 (128 x 12)
+//   16384 x 256 FP32 planes       97.0  90.5 (256 x 8)      FP64         888   838 (64 x 10)
+static void default_tile(lb_ctx* c) {
+  const int nx = c->grid.nx, ny = c->grid.ny, st = c->prm.storage;
+  const bool lg = c->prm.model == LB_MODEL_LIQUID_GAS;
+  int bx = 128, cols = 128, per_sm, most;  // CTAs per SM in one wave; tallest band
+  if (pull_storage(st)) {
+    // 30 columns a warp; a band also collides the two rows beside it, so taller bands
+    // on two thirds of the seven resident CTAs
+    cols = 120;
+    per_sm = 4;
+    most = 12;
+  } else if (!staged_ok(st, nx, ny)) {  // sliding window
+    per_sm = 4;
+    most = 16;
+  } else if (st == LB_STORAGE_F32_BLOCKED) {
+    per_sm = 4;
+    most = 8;
+  } else if (st == LB_STORAGE_F16_BLOCKED) {
+    per_sm = 5;
+    most = 12;
+  } else if (st == LB_STORAGE_F64) {
+    // the FP64 pipe bounds these: narrow tiles spread it evenly (binary: its stages
+    // leave two CTAs per SM, at twice the width)
+    bx = cols = lg ? 64 : 128;
+    per_sm = lg ? 8 : 2;
+    most = lg ? 10 : 12;
+  } else {
+    // planar storages: wide tiles, whose longer copies suit the copy engine, unless they
+    // leave SMs without a tile
+    bx = cols = (long)((nx + 255) / 256) * ny < device_sm_count() ? 128 : 256;
+    per_sm = bx == 256 ? 3 : 5;
+    most = lg ? 16 : (st == LB_STORAGE_F16DEV ? 12 : 8);
+  }
+  while (bx > 64 && nx <= bx / 2) {  // a narrow lattice: no idle half tiles
+    bx /= 2;
+    cols /= 2;
+    per_sm *= 2;
+  }
+  // rows of column blocks, less the solid share
+  const double rows = (double)((nx + cols - 1) / cols) * ((double)c->fluid / nx);
+  const double y = ceil(rows / ((double)per_sm * device_sm_count()));
+  c->tile_x = bx;
+  c->tile_y = y < most ? (y < 1 ? 1 : (int)y) : most;
+  if (c->tile_y > ny) c->tile_y = ny;
+}
+
 extern "C" {
 
 lb_status lb_create(const lb_grid* grid, const lb_walls* walls, const lb_params* params, const lb_alloc* alloc,
@@ -338,8 +396,6 @@ lb_status lb_create(const lb_grid* grid, const lb_walls* walls, const lb_params*
   c->have_alloc = alloc != NULL;
   if (alloc) c->alloc = *alloc;
   c->ops = pick_ops(params->model, params->storage);
-  c->tile_x = 128;
-  c->tile_y = grid->ny < 16 ? grid->ny : 16;
   c->gexec = NULL;
   c->err[0] = 0;
   if (cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess) {
@@ -389,6 +445,7 @@ lb_status lb_create(const lb_grid* grid, const lb_walls* walls, const lb_params*
   }
   // solid nodes: the tube's columns outside its band
   c->fluid = (long)grid->nx * grid->ny - (walls->tube_len > 0 ? (long)walls->tube_len * (grid->ny - walls->tube_h) : 0);
+  default_tile(c);
   st = default_state(c);
   if (st != LB_OK) {
     snprintf(g_create_err, sizeof g_create_err, "%s", c->err);
