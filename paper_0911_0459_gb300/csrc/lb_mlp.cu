@@ -2,16 +2,19 @@
 // kernels (include/lb_mlp.h).
 //
 // Contractions: C = A B on tensor cores, mma.sync m16n8k16 with BF16 operands
-// and FP32 accumulation.  A 64x64 tile per CTA (4 warps of 32x32), K in steps
-// of 16 staged through shared memory; operands are addressed through element
-// strides, so the transposed products of the backward pass need no copies.
+// and FP32 accumulation over K in steps of 16, from K = 0 upwards (every kernel
+// below keeps this order, so all of them give the same bits).  A 64x64 tile per CTA
+// (4 warps of 32x32); the operands come through a ring of cp.async stages of 64 K
+// values in 128-byte swizzled rows and leave it by ldmatrix, transposed where the
+// backward pass contracts over the rows of an array, so no operand is copied.
 // The weight gradients contract over the batch (K up to max_batch rows) into
-// small outputs: they split K over blockIdx.z and add the FP32 partials in a
-// fixed order afterwards (split-K, deterministic).
-// Epilogues fuse the bias and tanh (forward), the tanh derivative (backward)
-// and the BF16 rounding of activations.  Ensemble members run in the z
-// dimension of every launch.  One training iteration (forward, loss, backward,
-// AdamW) is captured once as a CUDA graph and replayed.
+// small outputs: they split K over CTAs, and the kernel that uses the gradient
+// adds the FP32 partials in a fixed order (split-K, deterministic).
+// Epilogues fuse the bias and tanh (forward), the loss and its derivative, the
+// tanh derivative (backward) and the BF16 rounding of activations.  Ensemble
+// members run in the z dimension of every launch.  One training iteration (forward,
+// loss, backward, AdamW: seven launches) is captured once as a CUDA graph and
+// replayed.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -29,26 +32,36 @@ namespace {
 
 typedef __nv_bfloat16 bf16;
 
-enum { EPI_F32 = 0, EPI_BIAS_F32 = 1, EPI_BIAS_TANH = 2, EPI_DTANH = 3 };
+constexpr int TM = 64, TN = 64, TK = 64;  // CTA tile; K values per stage
+constexpr int kGemmThreads = 128;
+constexpr int kStages = 3;
+constexpr int kTileBytes = TM * TK * 2;  // one operand of one stage (TM == TN)
+constexpr int kGemmSmem = kStages * 2 * kTileBytes;  // 48 KB: no opt-in, four CTAs per SM
+constexpr int kBiasGroups = 8;  // partial sums of a bias gradient (32 row classes each)
 
+enum { EPI_BIAS_F32 = 0, EPI_BIAS_TANH = 1, EPI_LOSS = 2, EPI_DTANH = 3, EPI_PART = 4 };
+
+// C (M x N) = A B over K rows [kb, ke).  Non-transposed operands hold K contiguous
+// (A[m][k], B[n][k]), transposed ones hold the other index contiguous (A[k][m],
+// B[k][n]); ld: elements per row, a multiple of 8, rows starting on 16 bytes.
 struct GemmArgs {
   int M, N, K;
   const bf16* A;
-  long sam, sak, a_mem;
+  long lda, a_mem;
   const bf16* B;
-  long sbk, sbn, b_mem;
-  int epi;
+  long ldb, b_mem;
+  int b_cols;  // transposed B: stored columns (>= N, a multiple of 8)
   const float* bias;
   long bias_mem;
-  float* Cf;
+  float* Cf;   // FP32 output, if any
   long ldcf, cf_mem;
-  bf16* Cb;
+  bf16* Cb;    // BF16 output, if any
   long ldcb, cb_mem;
   const bf16* H;  // activation whose tanh derivative multiplies (EPI_DTANH)
   long ldh, h_mem;
-  int ks;         // K splits: blockIdx.z = member * ks + split; split s takes K rows [s kc, (s + 1) kc)
-  int kc;
-  long cf_split;  // offset of split s's partial output from split 0's
+  const float* T;  // targets (EPI_LOSS) and the loss of every member
+  float* loss;
+  float scale;     // EPI_LOSS: 1 / (n n_out)
 };
 
 __device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
@@ -63,19 +76,214 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], const 
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-__global__ void __launch_bounds__(128) gemm_bf16_kernel(GemmArgs g) {
-  constexpr int TM = 64, TN = 64, TK = 16;
-  __shared__ bf16 As[TM][TK + 8];
-  __shared__ bf16 Bs[TK][TN + 8];
-  const int mem = blockIdx.z / g.ks, split = blockIdx.z - mem * g.ks;
-  const int kb = split * g.kc, ke = min(g.K, kb + g.kc);
-  const bf16* A = g.A + mem * g.a_mem;
-  const bf16* B = g.B + mem * g.b_mem;
-  const int m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+template <bool TRANS>
+__device__ __forceinline__ void ldmatrix4(uint32_t r[4], uint32_t addr) {
+  if constexpr (TRANS)
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+  else
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+// 16 bytes global -> shared, zeros when !ok (src is then not read)
+__device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Byte offset of 16-byte chunk c of row r in a stage of 128-byte rows: the chunks
+// of a row are permuted by its low three bits, so that the eight rows one ldmatrix
+// phase reads lie in different banks.
+__device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
+
+// One operand of one stage: 64 x 64 values.  Not transposed: rows are the output
+// index (from r0, below rmax), columns K (from k0, below ke, a multiple of 8 where
+// it ends the array).  Transposed: rows K, columns the output index (cmax).
+template <bool TRANS>
+__device__ __forceinline__ void stage_operand(uint32_t dst, const bf16* X, long ld, int r0, int rmax, int k0, int ke,
+                                              int tid) {
+#pragma unroll
+  for (int e = tid; e < 64 * 8; e += kGemmThreads) {
+    const int r = e >> 3, c = e & 7;
+    if constexpr (TRANS) {
+      const int k = k0 + r, m = r0 + 8 * c;
+      const bool ok = k < ke && m < rmax;
+      cp16(dst + swz(r, c), ok ? X + (long)k * ld + m : X, ok);
+    } else {
+      const int m = r0 + r, k = k0 + 8 * c;
+      const bool ok = m < rmax && k < ke;
+      cp16(dst + swz(r, c), ok ? X + (long)m * ld + k : X, ok);
+    }
+  }
+}
+
+// The 64x64 tile (m0, n0) of member mem, K rows [kb, ke), in the accumulators of
+// four warps (warp w: rows 32 (w / 2), columns 32 (w % 2)).
+template <bool TA, bool TB>
+__device__ __forceinline__ void gemm_tile(const bf16* A, long lda, int M, const bf16* B, long ldb, int bmax, int m0,
+                                          int n0, int kb, int ke, unsigned char* smem, float acc[2][4][4]) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+  const uint32_t sb = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.0f;
+  const int nk = (ke - kb + TK - 1) / TK;
+  auto load = [&](int c) {
+    if (c < nk) {
+      const uint32_t st = sb + (uint32_t)(c % kStages) * (2 * kTileBytes);
+      stage_operand<TA>(st, A, lda, m0, M, kb + c * TK, ke, tid);
+      stage_operand<TB>(st + kTileBytes, B, ldb, n0, bmax, kb + c * TK, ke, tid);
+    }
+    cp_commit();
+  };
+#pragma unroll
+  for (int c = 0; c < kStages - 1; ++c) load(c);
+  const int l8 = lane & 7, li = lane >> 3;
+  for (int c = 0; c < nk; ++c) {
+    cp_wait<kStages - 2>();
+    __syncthreads();
+    load(c + kStages - 1);
+    const uint32_t sa = sb + (uint32_t)(c % kStages) * (2 * kTileBytes), sbb = sa + kTileBytes;
+    const int left = ke - kb - c * TK;
+#pragma unroll
+    for (int ks = 0; ks < TK / 16; ++ks) {
+      if (ks * 16 >= left) break;
+      uint32_t a[2][4], b[2][4];
+#pragma unroll
+      for (int mi = 0; mi < 2; ++mi) {
+        if constexpr (TA)
+          ldmatrix4<true>(a[mi], sa + swz(ks * 16 + (li >> 1) * 8 + l8, ((wm + mi * 16) >> 3) + (li & 1)));
+        else
+          ldmatrix4<false>(a[mi], sa + swz(wm + mi * 16 + (li & 1) * 8 + l8, ks * 2 + (li >> 1)));
+      }
+#pragma unroll
+      for (int nj = 0; nj < 2; ++nj) {
+        if constexpr (TB)
+          ldmatrix4<true>(b[nj], sbb + swz(ks * 16 + (li & 1) * 8 + l8, ((wn + nj * 16) >> 3) + (li >> 1)));
+        else
+          ldmatrix4<false>(b[nj], sbb + swz(wn + nj * 16 + (li >> 1) * 8 + l8, ks * 2 + (li & 1)));
+      }
+#pragma unroll
+      for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+        for (int ni = 0; ni < 4; ++ni) mma_bf16(acc[mi][ni], a[mi], &b[ni >> 1][(ni & 1) * 2]);
+    }
+  }
+  cp_wait<0>();
+}
+
+// Store of the accumulators: f(m, n, v0, v1) for every pair of neighbouring columns
+// n, n + 1 inside the output (N is even, so a pair is inside as a whole).
+template <class F>
+__device__ __forceinline__ void for_pairs(const float acc[2][4][4], int m0, int n0, int M, int N, F f) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+  const int gq = lane >> 2, tq = lane & 3;
+#pragma unroll
+  for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int m = m0 + wm + mi * 16 + gq + h * 8;
+      if (m >= M) continue;
+#pragma unroll
+      for (int ni = 0; ni < 4; ++ni) {
+        const int n = n0 + wn + ni * 8 + 2 * tq;
+        if (n < N) f(m, n, acc[mi][ni][2 * h], acc[mi][ni][2 * h + 1]);
+      }
+    }
+}
+
+// Block sum of one value per thread, added to *out by thread 0 (sh: shared memory
+// that nothing else uses any more).
+__device__ __forceinline__ void block_add(float v, float scale, float* out, float* sh) {
+  __syncthreads();
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float s = 0.0f;
+    for (int w = 0; w < kGemmThreads / 32; ++w) s += sh[w];
+    atomicAdd(out, s * scale);
+  }
+}
+
+// Layers two and three and the backward products: grid (N tiles, M tiles, members).
+template <int EPI, bool TB>
+__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(GemmArgs g) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int mem = blockIdx.z, m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+  float acc[2][4][4];
+  gemm_tile<false, TB>(g.A + mem * g.a_mem, g.lda, g.M, g.B + mem * g.b_mem, g.ldb, TB ? g.b_cols : g.N, m0, n0, 0,
+                       g.K, smem, acc);
+  float* Cf = g.Cf ? g.Cf + mem * g.cf_mem : nullptr;
+  bf16* Cb = g.Cb ? g.Cb + mem * g.cb_mem : nullptr;
+  float sum = 0.0f;
+  for_pairs(acc, m0, n0, g.M, g.N, [&](int m, int n, float v0, float v1) {
+    if constexpr (EPI == EPI_BIAS_F32 || EPI == EPI_BIAS_TANH || EPI == EPI_LOSS) {
+      const float2 b = *reinterpret_cast<const float2*>(g.bias + mem * g.bias_mem + n);
+      v0 += b.x;
+      v1 += b.y;
+    }
+    if constexpr (EPI == EPI_BIAS_TANH) {
+      v0 = tanhf(v0);
+      v1 = tanhf(v1);
+    }
+    if constexpr (EPI == EPI_LOSS) {
+      // dY = 2 (Y - T) / (n n_out), and this tile's share of the loss
+      const float2 t = *reinterpret_cast<const float2*>(g.T + (long)m * g.N + n);
+      const float d0 = v0 - t.x, d1 = v1 - t.y;
+      sum += d0 * d0;
+      sum += d1 * d1;
+      v0 = 2.0f * d0 * g.scale;
+      v1 = 2.0f * d1 * g.scale;
+    }
+    if constexpr (EPI == EPI_DTANH) {
+      const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(g.H + mem * g.h_mem + (long)m * g.ldh + n);
+      const float h0 = __bfloat162float(h.x), h1 = __bfloat162float(h.y);
+      v0 *= 1.0f - h0 * h0;
+      v1 *= 1.0f - h1 * h1;
+    }
+    if (Cf) *reinterpret_cast<float2*>(Cf + (long)m * g.ldcf + n) = make_float2(v0, v1);
+    if (Cb)
+      *reinterpret_cast<uint32_t*>(Cb + (long)m * g.ldcb + n) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+  });
+  if constexpr (EPI == EPI_LOSS) block_add(sum, g.scale, g.loss + mem, reinterpret_cast<float*>(smem));
+}
+
+// Layer one: K = n_in <= 16 is one step of the tensor core, so the operands go
+// straight from global memory to registers (x is padded to 16 columns).  The first
+// CTA also clears the losses and counts the training step that begins.
+struct Sched {
+  int t;        // updates done, less one before the first
+  int total;    // length of the cosine schedule
+  float lr0, lr_min, wd;
+};
+__global__ void __launch_bounds__(kGemmThreads) layer1_kernel(const bf16* x, const bf16* w, long w_mem, const float* bias,
+                                                             long bias_mem, int n, int nin, int nh, bf16* h1,
+                                                             long h_mem, float* loss, int members, Sched* sc) {
+  const int mem = blockIdx.z, m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
+  if (sc && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
+    if (threadIdx.x < members) loss[threadIdx.x] = 0.0f;
+    if (threadIdx.x == 32) sc->t += 1;
+  }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
   const int gq = lane >> 2, tq = lane & 3;
   const bf16 zero = __float2bfloat16(0.0f);
+  const bf16* W = w + mem * w_mem;
   float acc[2][4][4];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
@@ -83,145 +291,178 @@ __global__ void __launch_bounds__(128) gemm_bf16_kernel(GemmArgs g) {
     for (int j = 0; j < 4; ++j)
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.0f;
-
-  for (int k0 = kb; k0 < ke; k0 += TK) {
-    // stage the A (TM x TK) and B (TK x TN) tiles; consecutive threads walk the
-    // unit-stride direction of each operand
-    for (int e = tid; e < TM * TK; e += 128) {
-      int r, c;
-      if (g.sam == 1) {
-        r = e % TM;
-        c = e / TM;
-      } else {
-        r = e / TK;
-        c = e % TK;
-      }
-      const int m = m0 + r, k = k0 + c;
-      As[r][c] = (m < g.M && k < ke) ? A[m * g.sam + k * g.sak] : zero;
-    }
-    for (int e = tid; e < TK * TN; e += 128) {
-      int r, c;
-      if (g.sbk == 1) {
-        r = e % TK;
-        c = e / TK;
-      } else {
-        r = e / TN;
-        c = e % TN;
-      }
-      const int k = k0 + r, n = n0 + c;
-      Bs[r][c] = (k < ke && n < g.N) ? B[k * g.sbk + n * g.sbn] : zero;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int mi = 0; mi < 2; ++mi) {
-      const int r = wm + mi * 16;
-      uint32_t a[4];
-      a[0] = pack2(As[r + gq][2 * tq], As[r + gq][2 * tq + 1]);
-      a[1] = pack2(As[r + gq + 8][2 * tq], As[r + gq + 8][2 * tq + 1]);
-      a[2] = pack2(As[r + gq][2 * tq + 8], As[r + gq][2 * tq + 9]);
-      a[3] = pack2(As[r + gq + 8][2 * tq + 8], As[r + gq + 8][2 * tq + 9]);
-#pragma unroll
-      for (int ni = 0; ni < 4; ++ni) {
-        const int c = wn + ni * 8 + gq;
-        uint32_t b[2];
-        b[0] = pack2(Bs[2 * tq][c], Bs[2 * tq + 1][c]);
-        b[1] = pack2(Bs[2 * tq + 8][c], Bs[2 * tq + 9][c]);
-        mma_bf16(acc[mi][ni], a, b);
-      }
-    }
-    __syncthreads();
-  }
-
-  const float* bias = g.bias ? g.bias + mem * g.bias_mem : nullptr;
-  float* Cf = g.Cf ? g.Cf + mem * g.cf_mem + split * g.cf_split : nullptr;
-  bf16* Cb = g.Cb ? g.Cb + mem * g.cb_mem : nullptr;
-  const bf16* H = g.H ? g.H + mem * g.h_mem : nullptr;
+  uint32_t a[2][4], b[4][2];
 #pragma unroll
   for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
-    for (int ni = 0; ni < 4; ++ni)
+    for (int q = 0; q < 4; ++q) {
+      const int m = m0 + wm + mi * 16 + gq + (q & 1) * 8;
+      a[mi][q] = m < n ? *reinterpret_cast<const uint32_t*>(x + (long)m * 16 + 2 * tq + (q >> 1) * 8) : 0u;
+    }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int m = m0 + wm + mi * 16 + gq + (q >> 1) * 8;
-        const int n = n0 + wn + ni * 8 + 2 * tq + (q & 1);
-        if (m >= g.M || n >= g.N) continue;
-        float v = acc[mi][ni][q];
-        if (g.epi == EPI_BIAS_F32 || g.epi == EPI_BIAS_TANH) v += bias[n];
-        if (g.epi == EPI_BIAS_TANH) v = tanhf(v);
-        if (g.epi == EPI_DTANH) {
-          const float h = __bfloat162float(H[(long)m * g.ldh + n]);
-          v *= 1.0f - h * h;
-        }
-        if (Cf) Cf[(long)m * g.ldcf + n] = v;
-        if (Cb) Cb[(long)m * g.ldcb + n] = __float2bfloat16(v);
-      }
+  for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int c = n0 + wn + ni * 8 + gq, k = 2 * tq + q * 8;
+      b[ni][q] = pack2(k < nin ? W[(long)c * nin + k] : zero, k + 1 < nin ? W[(long)c * nin + k + 1] : zero);
+    }
+#pragma unroll
+  for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+    for (int ni = 0; ni < 4; ++ni) mma_bf16(acc[mi][ni], a[mi], b[ni]);
+  bf16* H = h1 + mem * h_mem;
+  for_pairs(acc, m0, n0, n, nh, [&](int m, int c, float v0, float v1) {
+    const float2 bb = *reinterpret_cast<const float2*>(bias + mem * bias_mem + c);
+    v0 = tanhf(v0 + bb.x);
+    v1 = tanhf(v1 + bb.y);
+    *reinterpret_cast<uint32_t*>(H + (long)m * nh + c) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+  });
 }
 
-// dY = 2 (Y - T) / (n n_out) in FP32 and BF16; per-member loss accumulated.
-// out[m][n] (row stride ldo, member stride o_mem) = sum over s = 0 .. ks - 1, in that
-// order, of the split-K partials part[member][s][m][n] (dense M x N).
-__global__ void splitk_sum_kernel(const float* __restrict__ part, int ks, int M, int N, float* out, long ldo,
-                                  long o_mem) {
-  const int mem = blockIdx.y;
-  const long MN = (long)M * N;
-  const float* pm = part + (long)mem * ks * MN;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < MN; e += (long)gridDim.x * blockDim.x) {
-    float v = 0.0f;
-    for (int s = 0; s < ks; ++s) v += pm[s * MN + e];
-    out[mem * o_mem + (e / N) * ldo + (e % N)] = v;
-  }
-}
-
-__global__ void loss_grad_kernel(const float* Y, const float* T, int n, int nout, long mem_stride, float* dYf,
-                                 bf16* dYb, float* loss) {
-  const int mem = blockIdx.y;
-  const float scale = 1.0f / ((float)n * (float)nout);
-  float acc = 0.0f;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < (long)n * nout; e += (long)gridDim.x * blockDim.x) {
-    const float d = Y[mem * mem_stride + e] - T[e];
-    acc += d * d;
-    const float gr = 2.0f * d * scale;
-    dYf[mem * mem_stride + e] = gr;
-    dYb[mem * mem_stride + e] = __float2bfloat16(gr);
-  }
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  __shared__ float sh[32];
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.0f;
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) s += sh[w];
-    atomicAdd(&loss[mem], s * scale);
-  }
-}
-
-// out[mem][c] = sum over rows of X[mem][r][c] (bias gradients).
-__global__ void colsum_kernel(const float* X, int rows, int cols, long x_mem, float* out, long out_mem) {
-  const int mem = blockIdx.y;
-  const int c = blockIdx.x;
-  float acc = 0.0f;
-  for (int r = threadIdx.x; r < rows; r += blockDim.x) acc += X[mem * x_mem + (long)r * cols + c];
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  __shared__ float sh[32];
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float s = 0.0f;
-    for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) s += sh[w];
-    out[mem * out_mem + c] = s;
-  }
-}
-
-struct Sched {
-  int t;        // updates done
-  int total;    // length of the cosine schedule
-  float lr0, lr_min, wd;
+// Gradients of all weights and biases in one launch.  The first `tiles` blocks of
+// the grid's x take the 64x64 tiles of dW3, dW2 and dW1 for split y of the batch rows
+// (kc rows each); the others each take 32 columns of a bias gradient, for one of its
+// eight groups of row classes (y).  part: [member][split][P], at the parameters'
+// offsets; bpart: [member][group][b1 b2 b3].
+struct WgradArgs {
+  GemmArgs w[3];  // dW3 = dY^T H2, dW2 = dZ2^T H1, dW1 = dZ1^T X: A[k][m], B[k][n]
+  int tiles[3];   // tiles of each
+  int ntn[3];     // of them along N
+  int ks, kc;
+  const float* bx[3];  // dY, dZ2, dZ1 in FP32
+  int bcols[3];
+  int bblocks[3];      // blocks of 32 columns
+  int boff[3];         // offset of b3, b2, b1 in a bias partial
+  int bsum;            // 2 n_hidden + n_out
+  float* bpart;
+  int rows;
 };
 
-// AdamW on every member: FP32 master weights, BF16 working copy.  weight_mask
-// marks which parameter ranges are weights (decayed) and which are biases.
-__global__ void adamw_kernel(float* p, bf16* pb, const float* gr, float* m1, float* m2, long P, const Sched* sc,
-                             long b1, long w2, long b2, long w3, long b3) {
+// A bias gradient's column sums in the order of a 256-thread block whose thread t
+// adds rows t, t + 256, ... and whose warps reduce by xor shuffles: group y is warp y
+// of that block (row classes 32 y .. 32 y + 31).
+__device__ __forceinline__ void bias_group(const float* X, int rows, int cols, int c0, int grp, float* out,
+                                           float (*sh)[33]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = c0 + lane;
+  float s[8];
+#pragma unroll
+  for (int r = 0; r < 8; ++r) s[r] = 0.0f;
+  if (c < cols) {
+    const int t = grp * 32 + warp * 8;
+    int base = 0;
+    for (; base + t + 8 <= rows && base < rows; base += 256) {
+      float v[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = X[(long)(base + t + r) * cols + c];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) s[r] += v[r];
+    }
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+      if (base + t + r < rows) s[r] += X[(long)(base + t + r) * cols + c];
+  }
+#pragma unroll
+  for (int r = 0; r < 8; ++r) sh[warp * 8 + r][lane] = s[r];
+  for (int o = 16; o > 0; o >>= 1) {
+    __syncthreads();
+    for (int l = warp; l < o; l += kGemmThreads / 32) sh[l][lane] += sh[l + o][lane];
+  }
+  __syncthreads();
+  if (warp == 0 && c < cols) out[c] = sh[0][lane];
+}
+
+__global__ void __launch_bounds__(kGemmThreads) wgrad_kernel(WgradArgs a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  const int mem = blockIdx.z;
+  int t = blockIdx.x;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (t < a.tiles[q]) {
+      const int split = blockIdx.y;
+      if (split >= a.ks) return;
+      const GemmArgs& g = a.w[q];
+      const int m0 = t / a.ntn[q] * TM, n0 = t % a.ntn[q] * TN;
+      const int kb = split * a.kc, ke = min(g.K, kb + a.kc);
+      float acc[2][4][4];
+      gemm_tile<true, true>(g.A + mem * g.a_mem, g.lda, g.M, g.B + mem * g.b_mem, g.ldb, g.b_cols, m0, n0, kb, ke,
+                            smem, acc);
+      float* C = g.Cf + ((long)mem * a.ks + split) * g.cf_mem;
+      const int N = g.N;
+      for_pairs(acc, m0, n0, g.M, (N + 1) & ~1, [&](int m, int n, float v0, float v1) {
+        float* o = C + (long)m * N + n;
+        if (!(N & 1)) {
+          *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
+        } else {  // dW1 with an odd number of inputs
+          o[0] = v0;
+          if (n + 1 < N) o[1] = v1;
+        }
+      });
+      return;
+    }
+    t -= a.tiles[q];
+  }
+  if (blockIdx.y >= kBiasGroups) return;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    if (t < a.bblocks[q]) {
+      bias_group(a.bx[q] + mem * a.w[q].a_mem, a.rows, a.bcols[q], t * 32, blockIdx.y,
+                 a.bpart + ((long)mem * kBiasGroups + blockIdx.y) * a.bsum + a.boff[q],
+                 reinterpret_cast<float(*)[33]>(smem));
+      return;
+    }
+    t -= a.bblocks[q];
+  }
+}
+
+// Offsets of the parameter blocks (they and P are multiples of 8).
+struct Offsets {
+  long b1, w2, b2, w3, b3;
+  int nh, nout;
+};
+
+// The gradient of four neighbouring parameters of one member from its partials, in
+// split (weights) or group (biases) order.
+__device__ __forceinline__ float4 grad4(const float* part, const float* bpart, int ks, long P, const Offsets& o,
+                                        long i) {
+  const bool weight = (i < o.b1) || (i >= o.w2 && i < o.b2) || (i >= o.w3 && i < o.b3);
+  const float* p;
+  long stride;
+  int n;
+  if (weight) {
+    p = part + i;
+    stride = P;
+    n = ks;
+  } else {
+    const long c = i < o.w2 ? i - o.b1 : (i < o.w3 ? o.nh + (i - o.b2) : 2L * o.nh + (i - o.b3));
+    p = bpart + c;
+    stride = 2L * o.nh + o.nout;
+    n = kBiasGroups;
+  }
+  float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll 8
+  for (int s = 0; s < n; ++s) {
+    const float4 q = *reinterpret_cast<const float4*>(p + s * stride);
+    v.x += q.x;
+    v.y += q.y;
+    v.z += q.z;
+    v.w += q.w;
+  }
+  return v;
+}
+
+// Gradient of member blockIdx.y + mem0 into g (dense).
+__global__ void grad_sum_kernel(const float* part, const float* bpart, int ks, long P, Offsets o, int mem0, float* g) {
+  const long mem = mem0 + blockIdx.y;
+  for (long i = 4 * (blockIdx.x * (long)blockDim.x + threadIdx.x); i < P; i += 4L * gridDim.x * blockDim.x)
+    *reinterpret_cast<float4*>(g + mem * P + i) =
+        grad4(part + mem * ks * P, bpart + mem * kBiasGroups * (2L * o.nh + o.nout), ks, P, o, i);
+}
+
+// AdamW on every member, gradients straight from the partials: FP32 master weights,
+// BF16 working copy; the biases are not decayed.
+__global__ void __launch_bounds__(256) adamw_kernel(float* p, bf16* pb, const float* part, const float* bpart, int ks,
+                                                    float* m1, float* m2, long P, const Sched* sc, Offsets o) {
   const int mem = blockIdx.y;
   const int t = sc->t + 1;
   const float pi = 3.14159265358979f;
@@ -229,23 +470,34 @@ __global__ void adamw_kernel(float* p, bf16* pb, const float* gr, float* m1, flo
   const float lr = sc->lr_min + 0.5f * (sc->lr0 - sc->lr_min) * (1.0f + cosf(pi * frac));
   const float beta1 = 0.9f, beta2 = 0.999f, eps = 1e-8f;
   const float c1 = 1.0f - powf(beta1, (float)t), c2 = 1.0f - powf(beta2, (float)t);
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < P; i += (long)gridDim.x * blockDim.x) {
-    const long j = mem * P + i;
-    const float gv = gr[j];
-    const float a = beta1 * m1[j] + (1.0f - beta1) * gv;
-    const float b = beta2 * m2[j] + (1.0f - beta2) * gv * gv;
-    m1[j] = a;
-    m2[j] = b;
-    const bool weight = (i < b1) || (i >= w2 && i < b2) || (i >= w3 && i < b3);
-    float pv = p[j];
-    if (weight) pv -= lr * sc->wd * pv;
-    pv -= lr * (a / c1) / (sqrtf(b / c2) + eps);
-    p[j] = pv;
-    pb[j] = __float2bfloat16(pv);
+  const long i = 4 * (blockIdx.x * (long)blockDim.x + threadIdx.x);
+  if (i >= P) return;
+  const long j = mem * P + i;
+  const float4 g4 = grad4(part + (long)mem * ks * P, bpart + (long)mem * kBiasGroups * (2L * o.nh + o.nout), ks, P, o, i);
+  float4 a4 = *reinterpret_cast<float4*>(m1 + j), b4 = *reinterpret_cast<float4*>(m2 + j);
+  float4 p4 = *reinterpret_cast<float4*>(p + j);
+  const bool weight = (i < o.b1) || (i >= o.w2 && i < o.b2) || (i >= o.w3 && i < o.b3);
+  const float gr[4] = {g4.x, g4.y, g4.z, g4.w};
+  float av[4] = {a4.x, a4.y, a4.z, a4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w}, pv[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float gv = gr[q];
+    const float a = beta1 * av[q] + (1.0f - beta1) * gv;
+    const float b = beta2 * bv[q] + (1.0f - beta2) * gv * gv;
+    av[q] = a;
+    bv[q] = b;
+    float w = pv[q];
+    if (weight) w -= lr * sc->wd * w;
+    w -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+    pv[q] = w;
   }
+  *reinterpret_cast<float4*>(m1 + j) = make_float4(av[0], av[1], av[2], av[3]);
+  *reinterpret_cast<float4*>(m2 + j) = make_float4(bv[0], bv[1], bv[2], bv[3]);
+  *reinterpret_cast<float4*>(p + j) = make_float4(pv[0], pv[1], pv[2], pv[3]);
+  *reinterpret_cast<uint2*>(pb + j) =
+      make_uint2(pack2(__float2bfloat16(pv[0]), __float2bfloat16(pv[1])),
+                 pack2(__float2bfloat16(pv[2]), __float2bfloat16(pv[3])));
 }
-
-__global__ void advance_kernel(Sched* sc) { sc->t += 1; }
 
 // x (FP32, [n][n_in]) -> BF16 [n][16] with zero padding.
 __global__ void pack_x_kernel(const float* x, int n, int nin, bf16* xb) {
@@ -318,8 +570,8 @@ struct lb_mlp {
   // activations (per member)
   bf16 *xb, *xbp, *h1, *h2, *dyb, *dz2b, *dz1b;
   float *y, *dyf, *dz2f, *dz1f, *t;
-  float* part;  // split-K partials of the weight gradients
-  int ks_max;   // largest K split the partial buffer holds
+  float *part, *bpart;  // split-K partials of the weight gradients, row-class partials of the bias gradients
+  int ks_max;           // largest K split the partial buffer holds
   int n;  // rows of the loaded data
   cudaGraphExec_t gexec;
   int graph_n;
@@ -343,111 +595,175 @@ static void merr(lb_mlp* m, const char* fmt, ...) {
     }                                                                                      \
   } while (0)
 
+// Device memory on a 256-byte boundary (the kernels move 16 bytes at a time and an
+// allocator given by the caller may align to less).
 static void* malloc_dev(lb_mlp* m, size_t bytes) {
   void* p = NULL;
+  bytes += 256;
   if (m->have_alloc)
     p = m->alloc.malloc_fn(bytes, (void*)m->stream, m->alloc.user);
   else if (cudaMalloc(&p, bytes) != cudaSuccess) {
     cudaGetLastError();
     p = NULL;
   }
-  if (p) m->owned.push_back(p);
-  return p;
+  if (!p) return NULL;
+  m->owned.push_back(p);
+  return (void*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
 }
 
-static cudaError_t gemm(lb_mlp* m, cudaStream_t s, int M, int N, int K, const bf16* A, long sam, long sak,
-                        long a_mem, const bf16* B, long sbk, long sbn, long b_mem, int epi, const float* bias,
-                        long bias_mem, float* Cf, long ldcf, long cf_mem, bf16* Cb, long ldcb, long cb_mem,
-                        const bf16* H, long ldh, long h_mem) {
-  GemmArgs g = {M, N, K, A, sam, sak, a_mem, B, sbk, sbn, b_mem, epi, bias, bias_mem,
-                Cf, ldcf, cf_mem, Cb, ldcb, cb_mem, H, ldh, h_mem, 1, K, 0};
-  dim3 grid((N + 63) / 64, (M + 63) / 64, m->K);
-  gemm_bf16_kernel<<<grid, 128, 0, s>>>(g);
+// Release the newest allocation.
+static void free_last(lb_mlp* m) {
+  if (m->have_alloc)
+    m->alloc.free_fn(m->owned.back(), (void*)m->stream, m->alloc.user);
+  else
+    cudaFree(m->owned.back());
+  m->owned.pop_back();
+}
+
+template <int EPI, bool TB>
+static cudaError_t gemm(const GemmArgs& g, int members, cudaStream_t s) {
+  const dim3 grid((g.N + TN - 1) / TN, (g.M + TM - 1) / TM, members);
+  gemm_kernel<EPI, TB><<<grid, kGemmThreads, kGemmSmem, s>>>(g);
   return cudaGetLastError();
 }
 
-// A weight gradient C (M x N, FP32, row stride ldc, member stride c_mem) = A B with K
-// the batch: split-K over about 128 rows per split when K is long, then the fixed-order
-// sum of the partials into C.
-static cudaError_t gemm_wgrad(lb_mlp* m, cudaStream_t s, int M, int N, int K, const bf16* A, long sam, long sak,
-                              long a_mem, const bf16* B, long sbk, long sbn, long b_mem, float* C, long ldc,
-                              long c_mem) {
-  int ks = (K + 127) / 128;
-  if (ks > m->ks_max) ks = m->ks_max;
-  if (ks <= 1)
-    return gemm(m, s, M, N, K, A, sam, sak, a_mem, B, sbk, sbn, b_mem, EPI_F32, NULL, 0, C, ldc, c_mem, NULL, 0, 0,
-                NULL, 0, 0);
-  const int kc = ((K + ks - 1) / ks + 15) / 16 * 16;
-  ks = (K + kc - 1) / kc;
-  const long MN = (long)M * N;
-  GemmArgs g = {M, N, K, A, sam, sak, a_mem, B, sbk, sbn, b_mem, EPI_F32, NULL, 0,
-                m->part, N, ks * MN, NULL, 0, 0, NULL, 0, 0, ks, kc, MN};
-  dim3 grid((N + 63) / 64, (M + 63) / 64, m->K * ks);
-  gemm_bf16_kernel<<<grid, 128, 0, s>>>(g);
+// Forward of every member on rows [0, n) of the packed inputs xb: outputs in m->y, or
+// with train their loss against the loaded targets, and dY.
+static cudaError_t forward(lb_mlp* m, int n, const bf16* xb, bool train, cudaStream_t s) {
+  const long H = m->nh, O = m->nout, B = m->maxb;
+  layer1_kernel<<<dim3(m->nh / TN, (n + TM - 1) / TM, m->K), kGemmThreads, 0, s>>>(
+      xb, m->pb + m->ow1, m->P, m->p + m->ob1, m->P, n, m->nin, m->nh, m->h1, B * H, m->loss, m->K,
+      train ? m->sched : NULL);
   cudaError_t e = cudaGetLastError();
   if (e) return e;
-  const long blocks = (MN + 255) / 256;
-  splitk_sum_kernel<<<dim3((unsigned)(blocks < 1024 ? blocks : 1024), m->K), 256, 0, s>>>(m->part, ks, M, N, C, ldc,
-                                                                                          c_mem);
-  return cudaGetLastError();
+  GemmArgs g = {};
+  g.M = n;
+  g.N = m->nh;
+  g.K = m->nh;
+  g.A = m->h1;
+  g.lda = H;
+  g.a_mem = B * H;
+  g.B = m->pb + m->ow2;
+  g.ldb = H;
+  g.b_mem = m->P;
+  g.bias = m->p + m->ob2;
+  g.bias_mem = m->P;
+  g.Cb = m->h2;
+  g.ldcb = H;
+  g.cb_mem = B * H;
+  if ((e = gemm<EPI_BIAS_TANH, false>(g, m->K, s))) return e;
+  g.N = m->nout;
+  g.A = m->h2;
+  g.B = m->pb + m->ow3;
+  g.bias = m->p + m->ob3;
+  g.Cb = NULL;
+  g.Cf = m->y;
+  g.ldcf = O;
+  g.cf_mem = B * O;
+  if (!train) return gemm<EPI_BIAS_F32, false>(g, m->K, s);
+  g.Cf = m->dyf;
+  g.Cb = m->dyb;
+  g.ldcb = O;
+  g.cb_mem = B * O;
+  g.T = m->t;
+  g.loss = m->loss;
+  g.scale = 1.0f / ((float)n * (float)m->nout);
+  return gemm<EPI_LOSS, false>(g, m->K, s);
 }
 
-// forward of every member on rows [0, n) of the packed inputs xb; outputs in m->y
-static cudaError_t forward(lb_mlp* m, int n, const bf16* xb, cudaStream_t s) {
-  const long H = m->nh, O = m->nout, B = m->maxb;
-  cudaError_t e;
-  e = gemm(m, s, n, m->nh, m->nin, xb, 16, 1, 0, m->pb + m->ow1, 1, m->nin, m->P, EPI_BIAS_TANH, m->p + m->ob1, m->P,
-           NULL, 0, 0, m->h1, H, B * H, NULL, 0, 0);
-  if (e) return e;
-  e = gemm(m, s, n, m->nh, m->nh, m->h1, H, 1, B * H, m->pb + m->ow2, 1, H, m->P, EPI_BIAS_TANH, m->p + m->ob2, m->P,
-           NULL, 0, 0, m->h2, H, B * H, NULL, 0, 0);
-  if (e) return e;
-  return gemm(m, s, n, m->nout, m->nh, m->h2, H, 1, B * H, m->pb + m->ow3, 1, H, m->P, EPI_BIAS_F32, m->p + m->ob3,
-              m->P, m->y, O, B * O, NULL, 0, 0, NULL, 0, 0);
+// K splits of the weight gradients over n rows: about 128 rows each.
+static void wgrad_splits(const lb_mlp* m, int n, int* ks, int* kc) {
+  int k = (n + 127) / 128;
+  if (k > m->ks_max) k = m->ks_max;
+  *kc = k <= 1 ? n : ((n + k - 1) / k + 15) / 16 * 16;
+  *ks = (n + *kc - 1) / *kc;
 }
 
-// forward, loss and gradients of every member on the loaded data (grads in m->g)
+// forward, loss and the gradients' partials of every member on the loaded data
 static cudaError_t backward(lb_mlp* m, cudaStream_t s) {
   const int n = m->n;
   const long H = m->nh, O = m->nout, B = m->maxb;
-  cudaError_t e = forward(m, n, m->xb, s);
+  cudaError_t e = forward(m, n, m->xb, true, s);
   if (e) return e;
-  e = cudaMemsetAsync(m->loss, 0, m->K * sizeof(float), s);
-  if (e) return e;
-  loss_grad_kernel<<<dim3(64, m->K), 256, 0, s>>>(m->y, m->t, n, m->nout, B * O, m->dyf, m->dyb, m->loss);
-  if ((e = cudaGetLastError())) return e;
-  // dW3 = dY^T H2, db3 = colsum dY
-  e = gemm_wgrad(m, s, m->nout, m->nh, n, m->dyb, 1, O, B * O, m->h2, H, 1, B * H, m->g + m->ow3, H, m->P);
-  if (e) return e;
-  colsum_kernel<<<dim3(m->nout, m->K), 256, 0, s>>>(m->dyf, n, m->nout, B * O, m->g + m->ob3, m->P);
-  if ((e = cudaGetLastError())) return e;
-  // dZ2 = (dY W3) * (1 - H2^2)
-  e = gemm(m, s, n, m->nh, m->nout, m->dyb, O, 1, B * O, m->pb + m->ow3, H, 1, m->P, EPI_DTANH, NULL, 0, m->dz2f, H,
-           B * H, m->dz2b, H, B * H, m->h2, H, B * H);
-  if (e) return e;
-  // dW2 = dZ2^T H1, db2
-  e = gemm_wgrad(m, s, m->nh, m->nh, n, m->dz2b, 1, H, B * H, m->h1, H, 1, B * H, m->g + m->ow2, H, m->P);
-  if (e) return e;
-  colsum_kernel<<<dim3(m->nh, m->K), 256, 0, s>>>(m->dz2f, n, m->nh, B * H, m->g + m->ob2, m->P);
-  if ((e = cudaGetLastError())) return e;
-  // dZ1 = (dZ2 W2) * (1 - H1^2)
-  e = gemm(m, s, n, m->nh, m->nh, m->dz2b, H, 1, B * H, m->pb + m->ow2, H, 1, m->P, EPI_DTANH, NULL, 0, m->dz1f, H,
-           B * H, m->dz1b, H, B * H, m->h1, H, B * H);
-  if (e) return e;
-  // dW1 = dZ1^T X, db1
-  e = gemm_wgrad(m, s, m->nh, m->nin, n, m->dz1b, 1, H, B * H, m->xb, 16, 1, 0, m->g + m->ow1, m->nin, m->P);
-  if (e) return e;
-  colsum_kernel<<<dim3(m->nh, m->K), 256, 0, s>>>(m->dz1f, n, m->nh, B * H, m->g + m->ob1, m->P);
+  // dZ2 = (dY W3) * (1 - H2^2), dZ1 = (dZ2 W2) * (1 - H1^2)
+  GemmArgs g = {};
+  g.M = n;
+  g.N = m->nh;
+  g.K = m->nout;
+  g.A = m->dyb;
+  g.lda = O;
+  g.a_mem = B * O;
+  g.B = m->pb + m->ow3;
+  g.ldb = H;
+  g.b_mem = m->P;
+  g.b_cols = m->nh;
+  g.Cf = m->dz2f;
+  g.ldcf = H;
+  g.cf_mem = B * H;
+  g.Cb = m->dz2b;
+  g.ldcb = H;
+  g.cb_mem = B * H;
+  g.H = m->h2;
+  g.ldh = H;
+  g.h_mem = B * H;
+  if ((e = gemm<EPI_DTANH, true>(g, m->K, s))) return e;
+  g.K = m->nh;
+  g.A = m->dz2b;
+  g.lda = H;
+  g.a_mem = B * H;
+  g.B = m->pb + m->ow2;
+  g.Cf = m->dz1f;
+  g.Cb = m->dz1b;
+  g.H = m->h1;
+  if ((e = gemm<EPI_DTANH, true>(g, m->K, s))) return e;
+  // dW3 = dY^T H2, dW2 = dZ2^T H1, dW1 = dZ1^T X and the bias gradients
+  WgradArgs a = {};
+  const bf16* A[3] = {m->dyb, m->dz2b, m->dz1b};
+  const bf16* Bx[3] = {m->h2, m->h1, m->xb};
+  const int M[3] = {m->nout, m->nh, m->nh}, N[3] = {m->nh, m->nh, m->nin};
+  const long ow[3] = {m->ow3, m->ow2, m->ow1};
+  const float* bx[3] = {m->dyf, m->dz2f, m->dz1f};
+  int total = 0;
+  for (int q = 0; q < 3; ++q) {
+    GemmArgs& w = a.w[q];
+    w.M = M[q];
+    w.N = N[q];
+    w.K = n;
+    w.A = A[q];
+    w.lda = M[q];
+    w.a_mem = B * M[q];
+    w.B = Bx[q];
+    w.ldb = w.b_cols = q < 2 ? m->nh : 16;
+    w.b_mem = q < 2 ? B * H : 0;
+    w.Cf = m->part + ow[q];
+    w.cf_mem = m->P;
+    a.ntn[q] = (N[q] + TN - 1) / TN;
+    a.tiles[q] = (M[q] + TM - 1) / TM * a.ntn[q];
+    a.bx[q] = bx[q];
+    a.bcols[q] = M[q];
+    a.bblocks[q] = (M[q] + 31) / 32;
+    a.boff[q] = q == 0 ? 2 * m->nh : (q == 1 ? m->nh : 0);
+    total += a.tiles[q] + a.bblocks[q];
+  }
+  wgrad_splits(m, n, &a.ks, &a.kc);
+  a.bsum = 2 * m->nh + m->nout;
+  a.bpart = m->bpart;
+  a.rows = n;
+  wgrad_kernel<<<dim3(total, a.ks > kBiasGroups ? a.ks : kBiasGroups, m->K), kGemmThreads, kGemmSmem, s>>>(a);
   return cudaGetLastError();
+}
+
+static Offsets offsets(const lb_mlp* m) {
+  return Offsets{m->ob1, m->ow2, m->ob2, m->ow3, m->ob3, m->nh, m->nout};
 }
 
 static cudaError_t train_step(lb_mlp* m, cudaStream_t s) {
   cudaError_t e = backward(m, s);
   if (e) return e;
-  adamw_kernel<<<dim3(64, m->K), 256, 0, s>>>(m->p, m->pb, m->g, m->m1, m->m2, m->P, m->sched, m->ob1, m->ow2,
-                                               m->ob2, m->ow3, m->ob3);
-  if ((e = cudaGetLastError())) return e;
-  advance_kernel<<<1, 1, 0, s>>>(m->sched);
+  int ks, kc;
+  wgrad_splits(m, m->n, &ks, &kc);
+  adamw_kernel<<<dim3((unsigned)((m->P / 4 + 255) / 256), m->K), 256, 0, s>>>(m->p, m->pb, m->part, m->bpart, ks, m->m1,
+                                                                           m->m2, m->P, m->sched, offsets(m));
   return cudaGetLastError();
 }
 
@@ -495,8 +811,8 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
   m->dyf = (float*)malloc_dev(m, members * B * nout * 4);
   m->dyb = (bf16*)malloc_dev(m, members * B * nout * 2);
   m->t = (float*)malloc_dev(m, B * nout * 4);
-  // split-K partials of the largest weight gradient (nh x max(nh, nout)), about 128
-  // batch rows per split, at most 32 splits and 256 MB
+  // partials of the gradients: about 128 batch rows per split, at most 32 splits and,
+  // by the largest weight gradient (nh x max(nh, nout)), 256 MB
   {
     const long mn = (long)nh * (nh > nout ? nh : nout);
     long ks = (B + 127) / 128;
@@ -504,9 +820,10 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
     const long cap = (256L << 20) / (4L * members * mn);
     if (ks > cap) ks = cap;
     m->ks_max = ks > 1 ? (int)ks : 1;
-    m->part = m->ks_max > 1 ? (float*)malloc_dev(m, 4L * members * m->ks_max * mn) : NULL;
+    m->part = (float*)malloc_dev(m, 4L * members * m->ks_max * m->P);
+    m->bpart = (float*)malloc_dev(m, 4L * members * kBiasGroups * (2 * nh + nout));
   }
-  bool ok = (m->ks_max == 1 || m->part) && m->p && m->g && m->m1 && m->m2 && m->pb && m->sched && m->loss && m->xb && m->xbp && m->h1 && m->h2 && m->dz2b &&
+  bool ok = m->part && m->bpart && m->p && m->g && m->m1 && m->m2 && m->pb && m->sched && m->loss && m->xb && m->xbp && m->h1 && m->h2 && m->dz2b &&
             m->dz1b && m->dz2f && m->dz1f && m->y && m->dyf && m->dyb && m->t;
   if (!ok) {
     lb_mlp_destroy(m);
@@ -571,11 +888,7 @@ lb_status lb_mlp_set_data(lb_mlp* m, int n, const float* x, const float* y) {
   MCK(cudaGetLastError());
   MCK(cudaMemcpyAsync(m->t, y, (size_t)n * m->nout * 4, cudaMemcpyHostToDevice, m->stream));
   MCK(cudaStreamSynchronize(m->stream));
-  if (m->have_alloc)
-    m->alloc.free_fn(dx, (void*)m->stream, m->alloc.user);
-  else
-    cudaFree(dx);
-  m->owned.pop_back();
+  free_last(m);
   m->n = n;
   if (m->gexec) {
     cudaGraphExecDestroy(m->gexec);
@@ -587,6 +900,10 @@ lb_status lb_mlp_set_data(lb_mlp* m, int n, const float* x, const float* y) {
 lb_status lb_mlp_gradients(lb_mlp* m, int k, float* grads, float* loss) {
   if (!m || k < 0 || k >= m->K || !grads || m->n < 1) return LB_ERR_ARG;
   MCK(backward(m, m->stream));
+  int ks, kc;
+  wgrad_splits(m, m->n, &ks, &kc);
+  grad_sum_kernel<<<256, 256, 0, m->stream>>>(m->part, m->bpart, ks, m->P, offsets(m), k, m->g);
+  MCK(cudaGetLastError());
   MCK(cudaMemcpyAsync(grads, m->g + k * m->P, m->P * 4, cudaMemcpyDeviceToHost, m->stream));
   float hl[64];
   MCK(cudaMemcpyAsync(hl, m->loss, m->K * 4, cudaMemcpyDeviceToHost, m->stream));
@@ -597,7 +914,7 @@ lb_status lb_mlp_gradients(lb_mlp* m, int k, float* grads, float* loss) {
 
 lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, float* losses) {
   if (!m || steps < 1 || m->n < 1 || !(lr > 0)) return LB_ERR_ARG;
-  Sched sc = {0, steps, lr, lr_min, wd};
+  Sched sc = {-1, steps, lr, lr_min, wd};  // every step's first kernel counts it
   MCK(cudaMemcpyAsync(m->sched, &sc, sizeof sc, cudaMemcpyHostToDevice, m->stream));
   if (!m->gexec) {
     MCK(cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeThreadLocal));
@@ -612,7 +929,7 @@ lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, f
   for (int i = 0; i < steps; ++i) MCK(cudaGraphLaunch(m->gexec, m->stream));
   if (losses) {
     // loss of the final parameters
-    MCK(backward(m, m->stream));
+    MCK(forward(m, m->n, m->xb, true, m->stream));
     MCK(cudaMemcpyAsync(losses, m->loss, m->K * 4, cudaMemcpyDeviceToHost, m->stream));
   }
   MCK(cudaStreamSynchronize(m->stream));
@@ -629,7 +946,7 @@ lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* s
   MCK(cudaMemcpyAsync(dx, x, (size_t)n * m->nin * 4, cudaMemcpyHostToDevice, m->stream));
   pack_x_kernel<<<64, 256, 0, m->stream>>>(dx, n, m->nin, m->xbp);
   MCK(cudaGetLastError());
-  MCK(forward(m, n, m->xbp, m->stream));
+  MCK(forward(m, n, m->xbp, false, m->stream));
   ensemble_kernel<<<64, 256, 0, m->stream>>>(m->y, m->K, (long)m->maxb * m->nout, (long)n * m->nout, dmean, dsd);
   MCK(cudaGetLastError());
   MCK(cudaMemcpyAsync(mean, dmean, (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
@@ -639,11 +956,7 @@ lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* s
       MCK(cudaMemcpyAsync(members + (size_t)k * n * m->nout, m->y + (size_t)k * m->maxb * m->nout,
                           (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
   MCK(cudaStreamSynchronize(m->stream));
-  if (m->have_alloc)
-    m->alloc.free_fn(dx, (void*)m->stream, m->alloc.user);
-  else
-    cudaFree(dx);
-  m->owned.pop_back();
+  free_last(m);
   return LB_OK;
 }
 
