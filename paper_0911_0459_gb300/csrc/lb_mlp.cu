@@ -37,6 +37,9 @@ constexpr int kGemmThreads = 128;
 constexpr int kStages = 3;
 constexpr int kTileBytes = TM * TK * 2;  // one operand of one stage (TM == TN)
 constexpr int kGemmSmem = kStages * 2 * kTileBytes;  // 48 KB: no opt-in, four CTAs per SM
+constexpr int kWgradStages = 6;     // the weight gradients' long K: 96 KB in flight, two CTAs per SM
+constexpr int kWgradThreads = 128;  // four warps of 32x32 (eight of 32x16: 38 instead of 33 us)
+constexpr int kWgradSmem = kWgradStages * 2 * kTileBytes;
 constexpr int kBiasGroups = 8;  // partial sums of a bias gradient (32 row classes each)
 
 enum { EPI_BIAS_F32 = 0, EPI_BIAS_TANH = 1, EPI_LOSS = 2, EPI_DTANH = 3, EPI_PART = 4 };
@@ -90,7 +93,7 @@ __device__ __forceinline__ void ldmatrix4(uint32_t r[4], uint32_t addr) {
                  : "memory");
 }
 
-// 16 bytes global -> shared, zeros when !ok (src is then not read)
+// 16 bytes global -> shared, zeros when !ok (nothing is then read, wherever src points)
 __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool ok) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
 }
@@ -105,92 +108,157 @@ __device__ __forceinline__ void cp_wait() {
 // phase reads lie in different banks.
 __device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
 
-// One operand of one stage: 64 x 64 values.  Not transposed: rows are the output
-// index (from r0, below rmax), columns K (from k0, below ke, a multiple of 8 where
-// it ends the array).  Transposed: rows K, columns the output index (cmax).
-template <bool TRANS>
-__device__ __forceinline__ void stage_operand(uint32_t dst, const bf16* X, long ld, int r0, int rmax, int k0, int ke,
-                                              int tid) {
-#pragma unroll
-  for (int e = tid; e < 64 * 8; e += kGemmThreads) {
-    const int r = e >> 3, c = e & 7;
+// One operand of the ring: 64 x 64 values a stage, 16-byte chunks of NTH threads (rows
+// tid / 8 + NTH / 8 i, chunk tid % 8).  Not transposed: rows are the output index (from r0,
+// below rmax), columns K (a multiple of 8 ends the array).  Transposed: rows K, columns
+// the output index.  What a thread can know beforehand is kept here.
+template <bool TRANS, int NTH>
+struct Operand {
+  static constexpr int kRows = NTH / 8, kChunks = 64 / kRows;
+  const bf16* p;   // this thread's first chunk of the next stage
+  long step, row;  // elements to the next stage, and to the thread's next row
+  uint32_t dst;    // its place in a stage
+  int k;           // K index of the first chunk
+  unsigned in;     // bit i: chunk i's output index is inside
+  __device__ __forceinline__ Operand(const bf16* X, long ld, int r0, int rmax, int kb) {
+    const int r = threadIdx.x >> 3, c = threadIdx.x & 7;
+    dst = swz(r, c);
+    row = kRows * ld;
+    in = 0;
     if constexpr (TRANS) {
-      const int k = k0 + r, m = r0 + 8 * c;
-      const bool ok = k < ke && m < rmax;
-      cp16(dst + swz(r, c), ok ? X + (long)k * ld + m : X, ok);
+      k = kb + r;
+      p = X + (long)k * ld + r0 + 8 * c;
+      step = TK * ld;
+      if (r0 + 8 * c < rmax) in = 15u;
     } else {
-      const int m = r0 + r, k = k0 + 8 * c;
-      const bool ok = m < rmax && k < ke;
-      cp16(dst + swz(r, c), ok ? X + (long)m * ld + k : X, ok);
+      k = kb + 8 * c;
+      p = X + (long)(r0 + r) * ld + k;
+      step = TK;
+#pragma unroll
+      for (int i = 0; i < kChunks; ++i) in |= r0 + r + kRows * i < rmax ? 1u << i : 0u;
     }
   }
-}
+  __device__ __forceinline__ void stage(uint32_t base, int ke) {
+#pragma unroll
+    for (int i = 0; i < kChunks; ++i) {
+      cp16(base + dst + i * kRows * 128, p + i * row, (TRANS ? k + kRows * i < ke : k < ke) && (in >> i & 1u));
+    }
+    p += step;
+    k += TK;
+  }
+};
 
 // The 64x64 tile (m0, n0) of member mem, K rows [kb, ke), in the accumulators of
-// four warps (warp w: rows 32 (w / 2), columns 32 (w % 2)).
-template <bool TA, bool TB>
+// 2 WN warps (warp w: rows 32 (w / WN), 64 / WN columns from 64 / WN (w % WN)).  SPLIT: every kc rows the
+// accumulators are added to a running sum and start again from zero (kc a multiple of
+// 16 unless it covers the range).
+template <bool TA, bool TB, int WN = 2, int ST = kStages, bool SPLIT = false>
 __device__ __forceinline__ void gemm_tile(const bf16* A, long lda, int M, const bf16* B, long ldb, int bmax, int m0,
-                                          int n0, int kb, int ke, unsigned char* smem, float acc[2][4][4]) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+                                          int n0, int kb, int ke, unsigned char* smem, float acc[2][8 / WN][4],
+                                          int kc = 0) {
+  constexpr int NI = 8 / WN, NTH = 64 * WN;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int wm = (warp / WN) * 32, wn = (warp % WN) * (8 * NI);
   const uint32_t sb = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
 #pragma unroll
   for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int j = 0; j < NI; ++j)
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.0f;
   const int nk = (ke - kb + TK - 1) / TK;
+  Operand<TA, NTH> oa(A, lda, m0, M, kb);
+  Operand<TB, NTH> ob(B, ldb, n0, bmax, kb);
+  uint32_t wr = sb, rd = sb;  // the stages written and read next
   auto load = [&](int c) {
     if (c < nk) {
-      const uint32_t st = sb + (uint32_t)(c % kStages) * (2 * kTileBytes);
-      stage_operand<TA>(st, A, lda, m0, M, kb + c * TK, ke, tid);
-      stage_operand<TB>(st + kTileBytes, B, ldb, n0, bmax, kb + c * TK, ke, tid);
+      oa.stage(wr, ke);
+      ob.stage(wr + kTileBytes, ke);
+      wr = wr == sb + (ST - 1) * 2 * kTileBytes ? sb : wr + 2 * kTileBytes;
     }
     cp_commit();
   };
 #pragma unroll
-  for (int c = 0; c < kStages - 1; ++c) load(c);
+  for (int c = 0; c < ST - 1; ++c) load(c);
   const int l8 = lane & 7, li = lane >> 3;
-  for (int c = 0; c < nk; ++c) {
-    cp_wait<kStages - 2>();
-    __syncthreads();
-    load(c + kStages - 1);
-    const uint32_t sa = sb + (uint32_t)(c % kStages) * (2 * kTileBytes), sbb = sa + kTileBytes;
-    const int left = ke - kb - c * TK;
+  [[maybe_unused]] float run[2][NI][4];
+  [[maybe_unused]] int next = kc;  // rows after which the running sum takes the accumulators
+  if constexpr (SPLIT) {
 #pragma unroll
-    for (int ks = 0; ks < TK / 16; ++ks) {
-      if (ks * 16 >= left) break;
-      uint32_t a[2][4], b[2][4];
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < NI; ++j)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) run[i][j][k] = 0.0f;
+  }
+  for (int c = 0; c < nk; ++c) {
+    cp_wait<ST - 2>();
+    __syncthreads();
+    load(c + ST - 1);
+    const uint32_t sa = rd, sbb = rd + kTileBytes;
+    rd = rd == sb + (ST - 1) * 2 * kTileBytes ? sb : rd + 2 * kTileBytes;
+    const int steps = min((ke - kb - c * TK + 15) / 16, TK / 16);
+    uint32_t a[2][2][4], b[2][NI / 2][4];
+    auto frags = [&](int ks, int u) {
 #pragma unroll
       for (int mi = 0; mi < 2; ++mi) {
         if constexpr (TA)
-          ldmatrix4<true>(a[mi], sa + swz(ks * 16 + (li >> 1) * 8 + l8, ((wm + mi * 16) >> 3) + (li & 1)));
+          ldmatrix4<true>(a[u][mi], sa + swz(ks * 16 + (li >> 1) * 8 + l8, ((wm + mi * 16) >> 3) + (li & 1)));
         else
-          ldmatrix4<false>(a[mi], sa + swz(wm + mi * 16 + (li & 1) * 8 + l8, ks * 2 + (li >> 1)));
+          ldmatrix4<false>(a[u][mi], sa + swz(wm + mi * 16 + (li & 1) * 8 + l8, ks * 2 + (li >> 1)));
       }
 #pragma unroll
-      for (int nj = 0; nj < 2; ++nj) {
+      for (int nj = 0; nj < NI / 2; ++nj) {
         if constexpr (TB)
-          ldmatrix4<true>(b[nj], sbb + swz(ks * 16 + (li & 1) * 8 + l8, ((wn + nj * 16) >> 3) + (li >> 1)));
+          ldmatrix4<true>(b[u][nj], sbb + swz(ks * 16 + (li & 1) * 8 + l8, ((wn + nj * 16) >> 3) + (li >> 1)));
         else
-          ldmatrix4<false>(b[nj], sbb + swz(wn + nj * 16 + (li >> 1) * 8 + l8, ks * 2 + (li & 1)));
+          ldmatrix4<false>(b[u][nj], sbb + swz(wn + nj * 16 + (li >> 1) * 8 + l8, ks * 2 + (li & 1)));
       }
+    };
+    frags(0, 0);
+#pragma unroll
+    for (int ks = 0; ks < TK / 16; ++ks) {
+      if (ks >= steps) break;
+      if constexpr (SPLIT) {
+        if (c * TK + ks * 16 == next) {
+          next += kc;
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < NI; ++j)
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                run[i][j][k] += acc[i][j][k];
+                acc[i][j][k] = 0.0f;
+              }
+        }
+      }
+      if (ks + 1 < TK / 16) frags(ks + 1, (ks + 1) & 1);  // the next step's, while this one multiplies
 #pragma unroll
       for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
-        for (int ni = 0; ni < 4; ++ni) mma_bf16(acc[mi][ni], a[mi], &b[ni >> 1][(ni & 1) * 2]);
+        for (int ni = 0; ni < NI; ++ni)
+          mma_bf16(acc[mi][ni], a[ks & 1][mi], &b[ks & 1][ni >> 1][(ni & 1) * 2]);
     }
   }
   cp_wait<0>();
+  if constexpr (SPLIT) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < NI; ++j)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[i][j][k] = run[i][j][k] + acc[i][j][k];
+  }
 }
 
 // Store of the accumulators: f(m, n, v0, v1) for every pair of neighbouring columns
 // n, n + 1 inside the output (N is even, so a pair is inside as a whole).
-template <class F>
-__device__ __forceinline__ void for_pairs(const float acc[2][4][4], int m0, int n0, int M, int N, F f) {
+template <int WN = 2, class F>
+__device__ __forceinline__ void for_pairs(const float acc[2][8 / WN][4], int m0, int n0, int M, int N, F f) {
+  constexpr int NI = 8 / WN;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
+  const int wm = (warp / WN) * 32, wn = (warp % WN) * (8 * NI);
   const int gq = lane >> 2, tq = lane & 3;
 #pragma unroll
   for (int mi = 0; mi < 2; ++mi)
@@ -199,7 +267,7 @@ __device__ __forceinline__ void for_pairs(const float acc[2][4][4], int m0, int 
       const int m = m0 + wm + mi * 16 + gq + h * 8;
       if (m >= M) continue;
 #pragma unroll
-      for (int ni = 0; ni < 4; ++ni) {
+      for (int ni = 0; ni < NI; ++ni) {
         const int n = n0 + wn + ni * 8 + 2 * tq;
         if (n < N) f(m, n, acc[mi][ni][2 * h], acc[mi][ni][2 * h + 1]);
       }
@@ -264,21 +332,11 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(GemmArgs g) {
 }
 
 // Layer one: K = n_in <= 16 is one step of the tensor core, so the operands go
-// straight from global memory to registers (x is padded to 16 columns).  The first
-// CTA also clears the losses and counts the training step that begins.
-struct Sched {
-  int t;        // updates done, less one before the first
-  int total;    // length of the cosine schedule
-  float lr0, lr_min, wd;
-};
+// straight from global memory to registers (x is padded to 16 columns).
 __global__ void __launch_bounds__(kGemmThreads) layer1_kernel(const bf16* x, const bf16* w, long w_mem, const float* bias,
                                                              long bias_mem, int n, int nin, int nh, bf16* h1,
-                                                             long h_mem, float* loss, int members, Sched* sc) {
+                                                             long h_mem) {
   const int mem = blockIdx.z, m0 = blockIdx.y * TM, n0 = blockIdx.x * TN;
-  if (sc && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0) {
-    if (threadIdx.x < members) loss[threadIdx.x] = 0.0f;
-    if (threadIdx.x == 32) sc->t += 1;
-  }
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int wm = (warp >> 1) * 32, wn = (warp & 1) * 32;
   const int gq = lane >> 2, tq = lane & 3;
@@ -319,23 +377,373 @@ __global__ void __launch_bounds__(kGemmThreads) layer1_kernel(const bf16* x, con
   });
 }
 
-// Gradients of all weights and biases in one launch.  The first `tiles` blocks of
-// the grid's x take the 64x64 tiles of dW3, dW2 and dW1 for split y of the batch rows
-// (kc rows each); the others each take 32 columns of a bias gradient, for one of its
-// eight groups of row classes (y).  part: [member][split][P], at the parameters'
-// offsets; bpart: [member][group][b1 b2 b3].
+// ------------------------------------------------------------ fused row tiles
+//
+// Networks whose second weight matrix fits in shared memory (n_hidden <= 256): one
+// kernel takes a tile of 16 RT rows through all three layers and, when training,
+// through the loss and the backward products down to dZ1.  W2 and W3 stay in shared
+// memory while a CTA walks the tiles of a member (one CTA per SM, the tiles of all
+// members cut into equal runs), activations and upstream gradients never leave it
+// between layers, and what the weight gradients need goes to global memory as bulk
+// copies of whole rows behind the tensor-core work.  Against one GEMM launch per
+// product this saves the launches, the reloading of weights and activations per tile
+// and most of the address arithmetic; the tensor-core instructions and their order
+// along K are the same, so the results are too.  A warp takes all rows of the tile and
+// n_hidden / 8 columns, so that a weight fragment read from shared memory (whose
+// bandwidth is the bound) serves three products.  Rows of shared memory are padded by
+// 16 bytes: the eight rows of one ldmatrix phase then lie in different banks.
+// 4096 rows x 5 members, n_hidden 256, n_out 64: 46 us for the forward pass, the loss
+// and the backward products, against 85 us as five launches of the GEMM kernel above
+// (which takes the wider networks).  The tensor pipe is active a quarter of the time;
+// the rest is the FP32 gradients' stores, the tanh and the barriers between layers.
+struct RowsArgs {
+  int n, nin, nout, members;
+  const bf16* xb;    // packed inputs [n][16] (training)
+  const float* xf;   // inputs [n][n_in] (prediction)
+  const float* p;
+  const bf16* pb;
+  long P, ob1, ow2, ob2, ow3, ob3;
+  long B;            // rows between members in the activations
+  float* y;          // prediction
+  bf16 *h1, *h2, *dyb, *dz2b, *dz1b;
+  float *dyf, *dz2f, *dz1f;
+  const float* T;
+  float* loss;
+  float scale;
+};
+
+constexpr int kRowThreads = 256;  // eight warps (sixteen of half the columns: 49 instead of 47 us)
+
+// Shared memory of a row-tile CTA in bytes (o16: n_out rounded up to 16).
+constexpr size_t rows_smem(int nh, int nout, int rt, bool train) {
+  const size_t o16 = (nout + 15) / 16 * 16, ph = 2 * nh + 16;
+  return (nh + o16) * ph + 2 * 16 * rt * ph + (train ? 16 * rt * (2 * o16 + 16) : 0) + 64;
+}
+
+__device__ __forceinline__ void ldmatrix2(uint32_t r[2], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldmatrix2t(uint32_t r[2], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
+               : "=r"(r[0]), "=r"(r[1])
+               : "r"(addr)
+               : "memory");
+}
+// one row of shared memory to global memory by the copy engine (16-byte multiples)
+__device__ __forceinline__ void bulk_s2g(void* dst, uint32_t src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// acc (RT x NT fragments) = A[16 RT rows][K] B over K in steps of 16; A at sa with
+// pitch pa; B columns n0 .. n0 + 8 NT: rows n of pitch pb (not transposed) or rows k.
+template <int RT, int NT, bool TB>
+__device__ __forceinline__ void row_product(uint32_t sa, uint32_t pa, uint32_t sb, uint32_t pb, int n0, int K,
+                                            float acc[RT][NT][4]) {
+  const int lane = threadIdx.x & 31, l8 = lane & 7, li = lane >> 3;
+#pragma unroll
+  for (int i = 0; i < RT; ++i)
+#pragma unroll
+    for (int j = 0; j < NT; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0f;
+  const uint32_t aa = sa + ((li & 1) * 8 + l8) * pa + (li >> 1) * 16;
+  // not transposed: fragment pair j (columns 16 j, 16 j + 8) at rows n; transposed: at rows k
+  const uint32_t ba = TB ? sb + ((li & 1) * 8 + l8) * pb + 2 * n0 + (li >> 1) * 16
+                         : sb + (n0 + (li >> 1) * 8 + l8) * pb + (li & 1) * 16;
+  // fragments of step k + 16 are read while the tensor core works on step k
+  uint32_t a[2][RT][4], b[2][NT][2];
+  auto load = [&](int k, int u) {
+#pragma unroll
+    for (int i = 0; i < RT; ++i) ldmatrix4<false>(a[u][i], aa + i * 16 * pa + 2 * k);
+#pragma unroll
+    for (int j = 0; j < NT / 2; ++j) {
+      uint32_t r[4];
+      ldmatrix4<TB>(r, TB ? ba + k * pb + 32 * j : ba + 16 * j * pb + 2 * k);
+      b[u][2 * j][0] = r[0];
+      b[u][2 * j][1] = r[1];
+      b[u][2 * j + 1][0] = r[2];
+      b[u][2 * j + 1][1] = r[3];
+    }
+    if constexpr (NT & 1) {  // the last fragment alone (lanes 16..31's addresses are not used)
+      if constexpr (TB)
+        ldmatrix2t(b[u][NT - 1], sb + (k + (li & 1) * 8 + l8) * pb + 2 * (n0 + 8 * (NT - 1)));
+      else
+        ldmatrix2(b[u][NT - 1], sb + (n0 + 8 * (NT - 1) + l8) * pb + 2 * k + (li & 1) * 16);
+    }
+  };
+  auto multiply = [&](int u) {
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int j = 0; j < NT; ++j) mma_bf16(acc[i][j], a[u][i], b[u][j]);
+  };
+  load(0, 0);
+#pragma unroll 2
+  for (int k = 0; k < K; k += 32) {
+    if (k + 16 < K) load(k + 16, 1);
+    multiply(0);
+    if (k + 16 < K) {
+      if (k + 32 < K) load(k + 32, 0);
+      multiply(1);
+    }
+  }
+}
+
+template <int NT, int RT, bool TRAIN>
+__global__ void __launch_bounds__(kRowThreads, 1) rows_kernel(RowsArgs a) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int NF = NT;  // fragments of 8 columns per warp
+  constexpr int H = 64 * NT, R = 16 * RT;
+  constexpr uint32_t PH = 2 * H + 16;
+  const int O = a.nout, o16 = (O + 15) / 16 * 16, ot = O / 8;
+  const uint32_t PO = 2 * o16 + 16;
+  const uint32_t s0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
+  const uint32_t w2 = s0, w3 = w2 + H * PH, h1 = w3 + o16 * PH, h2 = h1 + R * PH, dy = h2 + R * PH;
+  unsigned char* const h1p = smem + (h1 - s0);
+  unsigned char* const h2p = smem + (h2 - s0);
+  unsigned char* const dyp = smem + (dy - s0);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gq = lane >> 2, tq = lane & 3;
+  const int nw = warp * 8 * NF;  // this warp's columns of the hidden layers
+  // this CTA's member and its run of the member's tiles
+  const int mem = blockIdx.x % a.members, slot = blockIdx.x / a.members, slots = gridDim.x / a.members;
+  const long per = (a.n + R - 1) / R;
+  const int t0 = (int)(per * slot / slots), t1 = (int)(per * (slot + 1) / slots);
+  float lsum = 0.0f;
+  {
+    const bf16* W2 = a.pb + mem * a.P + a.ow2;
+    const bf16* W3 = a.pb + mem * a.P + a.ow3;
+    for (int e = tid; e < (H + O) * (H / 8); e += kRowThreads) {
+      const int r = e / (H / 8), c = e % (H / 8);
+      cp16(w2 + r * PH + 16 * c, (r < H ? W2 + (long)r * H : W3 + (long)(r - H) * H) + 8 * c, true);
+    }
+    cp_commit();
+  }
+  // rows of W3 (and columns of dY) that only fill up the last step of 16
+  for (uint32_t e = tid; e < (o16 - O) * PH / 4; e += kRowThreads)
+    reinterpret_cast<uint32_t*>(smem + (w3 - s0) + O * PH)[e] = 0u;
+  uint32_t b1f[NF][2];
+  float2 bias1[NF], bias2[NF];
+  {
+    const bf16* W1 = a.pb + mem * a.P;
+    const bf16 zero = __float2bfloat16(0.0f);
+#pragma unroll
+    for (int j = 0; j < NF; ++j) {
+      const int c = nw + 8 * j + gq;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int k = 2 * tq + 8 * q;
+        b1f[j][q] = pack2(k < a.nin ? W1[(long)c * a.nin + k] : zero, k + 1 < a.nin ? W1[(long)c * a.nin + k + 1] : zero);
+      }
+      bias1[j] = *reinterpret_cast<const float2*>(a.p + mem * a.P + a.ob1 + nw + 8 * j + 2 * tq);
+      bias2[j] = *reinterpret_cast<const float2*>(a.p + mem * a.P + a.ob2 + nw + 8 * j + 2 * tq);
+    }
+  }
+  // the input fragments of a tile, read one tile ahead
+  uint32_t x[RT][4];
+  auto load_x = [&](int t) {
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int r = t * R + 16 * i + gq + (q & 1) * 8, k = 2 * tq + (q >> 1) * 8;
+        if constexpr (TRAIN) {
+          x[i][q] = r < a.n ? *reinterpret_cast<const uint32_t*>(a.xb + (long)r * 16 + k) : 0u;
+        } else {
+          const float* xr = a.xf + (long)r * a.nin;
+          x[i][q] = pack2(__float2bfloat16(r < a.n && k < a.nin ? xr[k] : 0.0f),
+                          __float2bfloat16(r < a.n && k + 1 < a.nin ? xr[k + 1] : 0.0f));
+        }
+      }
+  };
+  if (t0 < t1) load_x(t0);
+  for (int t = t0; t < t1; ++t) {
+    const int r0 = t * R;
+    const long row0 = mem * a.B + r0;  // first row of the tile in the activations
+    auto store_rows = [&](bf16* dst, uint32_t src, uint32_t pitch, int cols) {
+      if (tid < R && r0 + tid < a.n) bulk_s2g(dst + (row0 + tid) * cols, src + tid * pitch, 2 * cols);
+      if (tid < R) bulk_commit();
+    };
+    float acc[RT][NF][4];
+    // ---- layer 1: one tensor-core step from registers
+#pragma unroll
+    for (int i = 0; i < RT; ++i)
+#pragma unroll
+      for (int j = 0; j < NF; ++j) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0f;
+        mma_bf16(acc[i][j], x[i], b1f[j]);
+      }
+    if (t + 1 < t1) load_x(t + 1);
+    auto hidden = [&](unsigned char* dst, const float2 bias[NF]) {
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int j = 0; j < NF; ++j)
+            *reinterpret_cast<uint32_t*>(dst + (16 * i + 8 * h + gq) * PH + 2 * (nw + 8 * j + 2 * tq)) =
+                pack2(__float2bfloat16(tanhf(acc[i][j][2 * h] + bias[j].x)),
+                      __float2bfloat16(tanhf(acc[i][j][2 * h + 1] + bias[j].y)));
+    };
+    if constexpr (TRAIN) {
+      if (tid < R) bulk_wait_read();  // the last tile's copies out of these rows
+      __syncthreads();
+    }
+    hidden(h1p, bias1);
+    if constexpr (TRAIN) fence_async_smem();
+    cp_wait<0>();
+    __syncthreads();
+    if constexpr (TRAIN) store_rows(a.h1, h1, PH, H);
+    // ---- layer 2
+    row_product<RT, NF, false>(h1, PH, w2, PH, nw, H, acc);
+    hidden(h2p, bias2);
+    if constexpr (TRAIN) fence_async_smem();
+    __syncthreads();
+    if constexpr (TRAIN) store_rows(a.h2, h2, PH, H);
+    // ---- layer 3: eight columns per warp at a time
+    for (int c = warp; c < (TRAIN ? o16 / 8 : ot); c += kRowThreads / 32) {
+      if (c >= ot) {  // training: the padding of dY
+#pragma unroll
+        for (int i = 0; i < 2 * RT; ++i)
+          *reinterpret_cast<uint32_t*>(dyp + (8 * i + gq) * PO + 2 * (8 * c + 2 * tq)) = 0u;
+        continue;
+      }
+      float o3[RT][1][4];
+      const int n = 8 * c + 2 * tq;
+      [[maybe_unused]] float2 tt[RT][2];  // the targets, read while the product runs
+      if constexpr (TRAIN) {
+#pragma unroll
+        for (int i = 0; i < RT; ++i)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const int r = r0 + 16 * i + 8 * h + gq;
+            tt[i][h] = r < a.n ? *reinterpret_cast<const float2*>(a.T + (long)r * O + n) : make_float2(0.0f, 0.0f);
+          }
+      }
+      row_product<RT, 1, false>(h2, PH, w3, PH, 8 * c, H, o3);
+      const float2 b3 = *reinterpret_cast<const float2*>(a.p + mem * a.P + a.ob3 + n);
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = 16 * i + 8 * h + gq;
+          const bool in = r0 + r < a.n;
+          float v0 = o3[i][0][2 * h] + b3.x, v1 = o3[i][0][2 * h + 1] + b3.y;
+          if constexpr (!TRAIN) {
+            if (in) *reinterpret_cast<float2*>(a.y + (row0 + r) * O + n) = make_float2(v0, v1);
+          } else {
+            // dY = 2 (Y - T) / (n n_out)
+            float g0 = 0.0f, g1 = 0.0f;
+            if (in) {
+              const float d0 = v0 - tt[i][h].x, d1 = v1 - tt[i][h].y;
+              lsum += d0 * d0;
+              lsum += d1 * d1;
+              g0 = 2.0f * d0 * a.scale;
+              g1 = 2.0f * d1 * a.scale;
+              *reinterpret_cast<float2*>(a.dyf + (row0 + r) * O + n) = make_float2(g0, g1);
+            }
+            *reinterpret_cast<uint32_t*>(dyp + r * PO + 2 * n) = pack2(__float2bfloat16(g0), __float2bfloat16(g1));
+          }
+        }
+    }
+    if constexpr (!TRAIN) continue;
+    fence_async_smem();
+    if (tid < R) bulk_wait_read();  // h1 and h2 are rewritten below
+    __syncthreads();
+    store_rows(a.dyb, dy, PO, O);
+    // the products with (1 - h^2), over the activation's own place
+    auto dtanh = [&](unsigned char* hp, float* out) {
+#pragma unroll
+      for (int i = 0; i < RT; ++i)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = 16 * i + 8 * h + gq;
+#pragma unroll
+          for (int j = 0; j < NF; ++j) {
+            const int n = nw + 8 * j + 2 * tq;
+            __nv_bfloat162* q = reinterpret_cast<__nv_bfloat162*>(hp + r * PH + 2 * n);
+            const float h0 = __bfloat162float(q->x), h1v = __bfloat162float(q->y);
+            float v0 = acc[i][j][2 * h], v1 = acc[i][j][2 * h + 1];
+            v0 *= 1.0f - h0 * h0;
+            v1 *= 1.0f - h1v * h1v;
+            if (r0 + r < a.n) *reinterpret_cast<float2*>(out + (row0 + r) * H + n) = make_float2(v0, v1);
+            *reinterpret_cast<uint32_t*>(q) = pack2(__float2bfloat16(v0), __float2bfloat16(v1));
+          }
+        }
+    };
+    // ---- dZ2 = (dY W3) (1 - H2^2), dZ1 = (dZ2 W2) (1 - H1^2)
+    row_product<RT, NF, true>(dy, PO, w3, PH, nw, o16, acc);
+    dtanh(h2p, a.dz2f);
+    fence_async_smem();
+    __syncthreads();
+    store_rows(a.dz2b, h2, PH, H);
+    row_product<RT, NF, true>(h2, PH, w2, PH, nw, H, acc);
+    dtanh(h1p, a.dz1f);
+    fence_async_smem();
+    __syncthreads();
+    store_rows(a.dz1b, h1, PH, H);
+  }
+  if constexpr (TRAIN) {
+    for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+    if (lane == 0) atomicAdd(a.loss + mem, lsum * a.scale);
+    if (tid < R) bulk_wait_all();
+  }
+}
+
+template <int NT, int RT, bool TRAIN>
+static cudaError_t launch_rows_at(const RowsArgs& a, size_t smem, int sms, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(rows_kernel<NT, RT, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e) return e;
+  const long tiles = (a.n + 16 * RT - 1) / (16 * RT), slots = sms / a.members > 1 ? sms / a.members : 1;
+  rows_kernel<NT, RT, TRAIN><<<(unsigned)(a.members * (tiles < slots ? tiles : slots)), kRowThreads, smem, s>>>(a);
+  return cudaGetLastError();
+}
+template <int RT, bool TRAIN>
+static cudaError_t launch_rows_of(const RowsArgs& a, int nh, size_t smem, int sms, cudaStream_t s) {
+  switch (nh / 64) {
+    case 1: return launch_rows_at<1, RT, TRAIN>(a, smem, sms, s);
+    case 2: return launch_rows_at<2, RT, TRAIN>(a, smem, sms, s);
+    case 3: return launch_rows_at<3, RT, TRAIN>(a, smem, sms, s);
+    case 4: return launch_rows_at<4, RT, TRAIN>(a, smem, sms, s);
+  }
+  return cudaErrorInvalidValue;
+}
+template <bool TRAIN>
+static cudaError_t launch_rows(const RowsArgs& a, int nh, int rt, int sms, cudaStream_t s) {
+  const size_t smem = rows_smem(nh, a.nout, rt, TRAIN);
+  return rt == 3 ? launch_rows_of<3, TRAIN>(a, nh, smem, sms, s) : launch_rows_of<1, TRAIN>(a, nh, smem, sms, s);
+}
+
+// Gradients of all weights and biases in one launch.  The batch rows are cut into ks
+// splits of kc rows, whose products are added in split order.  Where the 64x64 tiles
+// of dW3, dW2 and dW1 fill the GPU by themselves a CTA takes a tile through all splits
+// and adds as it goes (parts = 1: no partial leaves the registers); otherwise the grid's
+// y is the split and the partials are added by the kernel that uses the gradient (parts
+// = ks).  The grid's x beyond the tiles takes 32 columns of a bias gradient each, for
+// one of its eight groups of row classes (y).  part: [member][parts][P], at the
+// parameters' offsets; bpart: [member][group][b1 b2 b3].
+struct Sched {
+  int t;        // updates done, less one before the first
+  int total;    // length of the cosine schedule
+  float lr0, lr_min, wd;
+};
 struct WgradArgs {
   GemmArgs w[3];  // dW3 = dY^T H2, dW2 = dZ2^T H1, dW1 = dZ1^T X: A[k][m], B[k][n]
   int tiles[3];   // tiles of each
   int ntn[3];     // of them along N
-  int ks, kc;
+  int ks, kc, parts;
   const float* bx[3];  // dY, dZ2, dZ1 in FP32
   int bcols[3];
   int bblocks[3];      // blocks of 32 columns
   int boff[3];         // offset of b3, b2, b1 in a bias partial
   int bsum;            // 2 n_hidden + n_out
   float* bpart;
-  int rows;
+  int rows, members;
+  Sched* sc;           // the training step this launch belongs to is counted here
 };
 
 // A bias gradient's column sums in the order of a 256-thread block whose thread t
@@ -345,70 +753,79 @@ __device__ __forceinline__ void bias_group(const float* X, int rows, int cols, i
                                            float (*sh)[33]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = c0 + lane;
-  float s[8];
+  constexpr int RC = 32 / (kWgradThreads / 32);  // row classes per warp
+  float s[RC];
 #pragma unroll
-  for (int r = 0; r < 8; ++r) s[r] = 0.0f;
+  for (int r = 0; r < RC; ++r) s[r] = 0.0f;
   if (c < cols) {
-    const int t = grp * 32 + warp * 8;
-    int base = 0;
-    for (; base + t + 8 <= rows && base < rows; base += 256) {
-      float v[8];
+    const int t = grp * 32 + warp * RC;
+    const float* p = X + (long)t * cols + c;
+    const long step = 256L * cols;
+    int base = t + RC;
+#pragma unroll 4
+    for (; base <= rows; base += 256, p += step) {
 #pragma unroll
-      for (int r = 0; r < 8; ++r) v[r] = X[(long)(base + t + r) * cols + c];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) s[r] += v[r];
+      for (int r = 0; r < RC; ++r) s[r] += p[r * cols];
     }
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
-      if (base + t + r < rows) s[r] += X[(long)(base + t + r) * cols + c];
+    for (int r = 0; r < RC; ++r)
+      if (base - RC + r < rows) s[r] += p[r * cols];
   }
 #pragma unroll
-  for (int r = 0; r < 8; ++r) sh[warp * 8 + r][lane] = s[r];
+  for (int r = 0; r < RC; ++r) sh[warp * RC + r][lane] = s[r];
   for (int o = 16; o > 0; o >>= 1) {
     __syncthreads();
-    for (int l = warp; l < o; l += kGemmThreads / 32) sh[l][lane] += sh[l + o][lane];
+    for (int l = warp; l < o; l += kWgradThreads / 32) sh[l][lane] += sh[l + o][lane];
   }
   __syncthreads();
   if (warp == 0 && c < cols) out[c] = sh[0][lane];
 }
 
-__global__ void __launch_bounds__(kGemmThreads) wgrad_kernel(WgradArgs a) {
+__global__ void __launch_bounds__(kWgradThreads) wgrad_kernel(WgradArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
-  const int mem = blockIdx.z;
+  if (a.sc && blockIdx.x == 0 && threadIdx.x == 0) a.sc->t += 1;
+  // the products first (they take longest): member, then split, then tile
   int t = blockIdx.x;
+  const int nprod = (a.tiles[0] + a.tiles[1] + a.tiles[2]) * a.parts * a.members;
+  const bool prod = t < nprod;
+  if (!prod) t -= nprod;
+  const int mem = t % a.members;
+  t /= a.members;
+  const int ny = prod ? a.parts : kBiasGroups;
+  const int y = t % ny;  // split or group
+  t /= ny;
+  if (prod) {
 #pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    if (t < a.tiles[q]) {
-      const int split = blockIdx.y;
-      if (split >= a.ks) return;
-      const GemmArgs& g = a.w[q];
-      const int m0 = t / a.ntn[q] * TM, n0 = t % a.ntn[q] * TN;
-      const int kb = split * a.kc, ke = min(g.K, kb + a.kc);
-      float acc[2][4][4];
-      gemm_tile<true, true>(g.A + mem * g.a_mem, g.lda, g.M, g.B + mem * g.b_mem, g.ldb, g.b_cols, m0, n0, kb, ke,
-                            smem, acc);
-      float* C = g.Cf + ((long)mem * a.ks + split) * g.cf_mem;
-      const int N = g.N;
-      for_pairs(acc, m0, n0, g.M, (N + 1) & ~1, [&](int m, int n, float v0, float v1) {
-        float* o = C + (long)m * N + n;
-        if (!(N & 1)) {
-          *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
-        } else {  // dW1 with an odd number of inputs
-          o[0] = v0;
-          if (n + 1 < N) o[1] = v1;
-        }
-      });
-      return;
+    for (int q = 0; q < 3; ++q) {
+      if (t < a.tiles[q]) {
+        const GemmArgs& g = a.w[q];
+        const int m0 = t / a.ntn[q] * TM, n0 = t % a.ntn[q] * TN;
+        const int kb = y * a.kc, ke = a.parts == 1 ? g.K : min(g.K, kb + a.kc);
+        float acc[2][4][4];
+        gemm_tile<true, true, 2, kWgradStages, true>(g.A + mem * g.a_mem, g.lda, g.M, g.B + mem * g.b_mem, g.ldb, g.b_cols,
+                                                  m0, n0, kb, ke, smem, acc, a.kc);
+        float* C = g.Cf + ((long)mem * a.parts + y) * g.cf_mem;
+        const int N = g.N;
+        for_pairs<2>(acc, m0, n0, g.M, (N + 1) & ~1, [&](int m, int n, float v0, float v1) {
+          float* o = C + (long)m * N + n;
+          if (!(N & 1)) {
+            *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
+          } else {  // dW1 with an odd number of inputs
+            o[0] = v0;
+            if (n + 1 < N) o[1] = v1;
+          }
+        });
+        return;
+      }
+      t -= a.tiles[q];
     }
-    t -= a.tiles[q];
+    return;
   }
-  if (blockIdx.y >= kBiasGroups) return;
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     if (t < a.bblocks[q]) {
-      bias_group(a.bx[q] + mem * a.w[q].a_mem, a.rows, a.bcols[q], t * 32, blockIdx.y,
-                 a.bpart + ((long)mem * kBiasGroups + blockIdx.y) * a.bsum + a.boff[q],
-                 reinterpret_cast<float(*)[33]>(smem));
+      bias_group(a.bx[q] + mem * a.w[q].a_mem, a.rows, a.bcols[q], t * 32, y,
+                 a.bpart + ((long)mem * kBiasGroups + y) * a.bsum + a.boff[q], reinterpret_cast<float(*)[33]>(smem));
       return;
     }
     t -= a.bblocks[q];
@@ -462,8 +879,10 @@ __global__ void grad_sum_kernel(const float* part, const float* bpart, int ks, l
 // AdamW on every member, gradients straight from the partials: FP32 master weights,
 // BF16 working copy; the biases are not decayed.
 __global__ void __launch_bounds__(256) adamw_kernel(float* p, bf16* pb, const float* part, const float* bpart, int ks,
-                                                    float* m1, float* m2, long P, const Sched* sc, Offsets o) {
+                                                    float* m1, float* m2, long P, const Sched* sc, Offsets o,
+                                                    float* loss) {
   const int mem = blockIdx.y;
+  if (blockIdx.x == 0 && threadIdx.x == 0) loss[mem] = 0.0f;  // for the next step
   const int t = sc->t + 1;
   const float pi = 3.14159265358979f;
   const float frac = sc->total > 1 ? fminf((float)(t - 1) / (float)(sc->total - 1), 1.0f) : 1.0f;
@@ -497,6 +916,19 @@ __global__ void __launch_bounds__(256) adamw_kernel(float* p, bf16* pb, const fl
   *reinterpret_cast<uint2*>(pb + j) =
       make_uint2(pack2(__float2bfloat16(pv[0]), __float2bfloat16(pv[1])),
                  pack2(__float2bfloat16(pv[2]), __float2bfloat16(pv[3])));
+}
+
+// A member's new master weights: the BF16 working copy, and fresh AdamW moments (the
+// host's own conversion of 83520 weights took 140 us a member, this takes 26 with the copy).
+__global__ void __launch_bounds__(256) load_params_kernel(const float* p, bf16* pb, float* m1, float* m2, long P) {
+  const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  for (long i = 4 * (blockIdx.x * (long)blockDim.x + threadIdx.x); i < P; i += 4L * gridDim.x * blockDim.x) {
+    const float4 v = *reinterpret_cast<const float4*>(p + i);
+    *reinterpret_cast<uint2*>(pb + i) = make_uint2(pack2(__float2bfloat16(v.x), __float2bfloat16(v.y)),
+                                                   pack2(__float2bfloat16(v.z), __float2bfloat16(v.w)));
+    *reinterpret_cast<float4*>(m1 + i) = z;
+    *reinterpret_cast<float4*>(m2 + i) = z;
+  }
 }
 
 // x (FP32, [n][n_in]) -> BF16 [n][16] with zero padding.
@@ -535,19 +967,33 @@ __global__ void init_params_kernel(float* p, bf16* pb, long P, unsigned long lon
   }
 }
 
-// mean and standard deviation over members of Y [K][n][nout].
-__global__ void ensemble_kernel(const float* Y, int K, long stride, long count, float* mean, float* sd) {
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < count; e += (long)gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int k = 0; k < K; ++k) s += Y[k * stride + e];
-    const float mu = s / K;
-    float q = 0.0f;
+// mean and standard deviation over members of Y [K][n][nout], four values at a time
+// (count, the member stride and the arrays are multiples of 16 bytes).
+__global__ void __launch_bounds__(256) ensemble_kernel(const float* Y, int K, long stride, long count, float* mean,
+                                                       float* sd) {
+  for (long e = 4 * (blockIdx.x * (long)blockDim.x + threadIdx.x); e < count; e += 4L * gridDim.x * blockDim.x) {
+    float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, q[4] = {0.0f, 0.0f, 0.0f, 0.0f}, mu[4], dv[4];
     for (int k = 0; k < K; ++k) {
-      const float d = Y[k * stride + e] - mu;
-      q += d * d;
+      const float4 v = *reinterpret_cast<const float4*>(Y + k * stride + e);
+      const float y[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) s[i] += y[i];
     }
-    mean[e] = mu;
-    sd[e] = K > 1 ? sqrtf(q / (K - 1)) : 0.0f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) mu[i] = s[i] / K;
+    for (int k = 0; k < K; ++k) {
+      const float4 v = *reinterpret_cast<const float4*>(Y + k * stride + e);
+      const float y[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float d = y[i] - mu[i];
+        q[i] += d * d;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dv[i] = K > 1 ? sqrtf(q[i] / (K - 1)) : 0.0f;
+    *reinterpret_cast<float4*>(mean + e) = make_float4(mu[0], mu[1], mu[2], mu[3]);
+    *reinterpret_cast<float4*>(sd + e) = make_float4(dv[0], dv[1], dv[2], dv[3]);
   }
 }
 
@@ -573,6 +1019,9 @@ struct lb_mlp {
   float *part, *bpart;  // split-K partials of the weight gradients, row-class partials of the bias gradients
   int ks_max;           // largest K split the partial buffer holds
   int n;  // rows of the loaded data
+  int sms;          // SMs of the device and shared memory a block may opt in to
+  size_t max_smem;
+  float *xin, *mean, *sd;  // host rows on their way in, ensemble statistics on their way out
   cudaGraphExec_t gexec;
   int graph_n;
   char err[512];
@@ -611,13 +1060,10 @@ static void* malloc_dev(lb_mlp* m, size_t bytes) {
   return (void*)(((uintptr_t)p + 255) & ~(uintptr_t)255);
 }
 
-// Release the newest allocation.
-static void free_last(lb_mlp* m) {
-  if (m->have_alloc)
-    m->alloc.free_fn(m->owned.back(), (void*)m->stream, m->alloc.user);
-  else
-    cudaFree(m->owned.back());
-  m->owned.pop_back();
+// Blocks of 256 threads for a grid-stride kernel over count items.
+static unsigned blocks_for(const lb_mlp* m, long count) {
+  const long b = (count + 255) / 256, most = 16L * m->sms;
+  return (unsigned)(b < 1 ? 1 : (b < most ? b : most));
 }
 
 template <int EPI, bool TB>
@@ -627,13 +1073,50 @@ static cudaError_t gemm(const GemmArgs& g, int members, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Forward of every member on rows [0, n) of the packed inputs xb: outputs in m->y, or
-// with train their loss against the loaded targets, and dY.
+// Rows in units of 16 that a fused row tile takes (0: the network does not fit): three
+// where the tiles of 48 rows still give every SM one, else one, so that small batches
+// spread over the SMs (512 rows x 5 members: 160 tiles of 16 rows).
+static int rows_plan(const lb_mlp* m, int n, bool train) {
+  if (m->nh > 256) return 0;
+  if ((long)((n + 47) / 48) * m->K >= m->sms && rows_smem(m->nh, m->nout, 3, train) <= m->max_smem) return 3;
+  return rows_smem(m->nh, m->nout, 1, train) <= m->max_smem ? 1 : 0;
+}
+
+static RowsArgs rows_args(const lb_mlp* m, int n) {
+  RowsArgs a = {};
+  a.n = n; a.nin = m->nin; a.nout = m->nout; a.members = m->K;
+  a.p = m->p; a.pb = m->pb; a.P = m->P;
+  a.ob1 = m->ob1; a.ow2 = m->ow2; a.ob2 = m->ob2; a.ow3 = m->ow3; a.ob3 = m->ob3;
+  a.B = m->maxb;
+  return a;
+}
+
+// The fused forward and backward pass of the loaded data down to dZ1.
+static cudaError_t rows_train(lb_mlp* m, int rt, cudaStream_t s) {
+  RowsArgs a = rows_args(m, m->n);
+  a.xb = m->xb;
+  a.h1 = m->h1; a.h2 = m->h2; a.dyb = m->dyb; a.dz2b = m->dz2b; a.dz1b = m->dz1b;
+  a.dyf = m->dyf; a.dz2f = m->dz2f; a.dz1f = m->dz1f;
+  a.T = m->t;
+  a.loss = m->loss;
+  a.scale = 1.0f / ((float)m->n * (float)m->nout);
+  return launch_rows<true>(a, m->nh, rt, m->sms, s);
+}
+
+// Forward of every member on n rows of inputs x: outputs in m->y.
+static cudaError_t rows_predict(lb_mlp* m, int rt, int n, const float* x, cudaStream_t s) {
+  RowsArgs a = rows_args(m, n);
+  a.xf = x;
+  a.y = m->y;
+  return launch_rows<false>(a, m->nh, rt, m->sms, s);
+}
+
+// One launch per product.  Forward of every member on rows [0, n) of the packed inputs
+// xb: outputs in m->y, or with train their loss against the loaded targets, and dY.
 static cudaError_t forward(lb_mlp* m, int n, const bf16* xb, bool train, cudaStream_t s) {
   const long H = m->nh, O = m->nout, B = m->maxb;
   layer1_kernel<<<dim3(m->nh / TN, (n + TM - 1) / TM, m->K), kGemmThreads, 0, s>>>(
-      xb, m->pb + m->ow1, m->P, m->p + m->ob1, m->P, n, m->nin, m->nh, m->h1, B * H, m->loss, m->K,
-      train ? m->sched : NULL);
+      xb, m->pb + m->ow1, m->P, m->p + m->ob1, m->P, n, m->nin, m->nh, m->h1, B * H);
   cudaError_t e = cudaGetLastError();
   if (e) return e;
   GemmArgs g = {};
@@ -679,8 +1162,8 @@ static void wgrad_splits(const lb_mlp* m, int n, int* ks, int* kc) {
   *ks = (n + *kc - 1) / *kc;
 }
 
-// forward, loss and the gradients' partials of every member on the loaded data
-static cudaError_t backward(lb_mlp* m, cudaStream_t s) {
+// Forward, loss and backward products of every member on the loaded data, one launch each.
+static cudaError_t gemm_train(lb_mlp* m, cudaStream_t s) {
   const int n = m->n;
   const long H = m->nh, O = m->nout, B = m->maxb;
   cudaError_t e = forward(m, n, m->xb, true, s);
@@ -715,15 +1198,34 @@ static cudaError_t backward(lb_mlp* m, cudaStream_t s) {
   g.Cf = m->dz1f;
   g.Cb = m->dz1b;
   g.H = m->h1;
-  if ((e = gemm<EPI_DTANH, true>(g, m->K, s))) return e;
+  return gemm<EPI_DTANH, true>(g, m->K, s);
+}
+
+// Parts the weight gradients are left in: 1 where the tiles fill three quarters of the
+// SMs, or where a CTA's pass over all rows is short, else one per split.  4096 rows x 5
+// members (120 tiles): 38 us in one part, 41 us in 32 parts and 2 us more in AdamW, which
+// then reads 54 MB of partials; one member alone (24 tiles) needs the splits to fill the SMs.
+static int wgrad_parts(const lb_mlp* m, int ks) {
+  const long h = m->nh / TM, o = (m->nout + TM - 1) / TM;
+  return ks <= 4 || 4 * (h * h + h * o + h) * m->K >= 3 * m->sms ? 1 : ks;
+}
+
+// forward, loss and the gradients' partials of every member on the loaded data (sc:
+// the schedule that counts training steps, or NULL); the losses are added to m->loss
+static cudaError_t backward(lb_mlp* m, Sched* sc, cudaStream_t s) {
+  const int n = m->n;
+  const long H = m->nh, B = m->maxb;
+  const int rt = rows_plan(m, m->n, true);
+  cudaError_t e = rt ? rows_train(m, rt, s) : gemm_train(m, s);
+  if (e) return e;
   // dW3 = dY^T H2, dW2 = dZ2^T H1, dW1 = dZ1^T X and the bias gradients
   WgradArgs a = {};
+  a.sc = sc;
   const bf16* A[3] = {m->dyb, m->dz2b, m->dz1b};
   const bf16* Bx[3] = {m->h2, m->h1, m->xb};
   const int M[3] = {m->nout, m->nh, m->nh}, N[3] = {m->nh, m->nh, m->nin};
   const long ow[3] = {m->ow3, m->ow2, m->ow1};
   const float* bx[3] = {m->dyf, m->dz2f, m->dz1f};
-  int total = 0;
   for (int q = 0; q < 3; ++q) {
     GemmArgs& w = a.w[q];
     w.M = M[q];
@@ -743,13 +1245,18 @@ static cudaError_t backward(lb_mlp* m, cudaStream_t s) {
     a.bcols[q] = M[q];
     a.bblocks[q] = (M[q] + 31) / 32;
     a.boff[q] = q == 0 ? 2 * m->nh : (q == 1 ? m->nh : 0);
-    total += a.tiles[q] + a.bblocks[q];
   }
   wgrad_splits(m, n, &a.ks, &a.kc);
+  a.parts = wgrad_parts(m, a.ks);
   a.bsum = 2 * m->nh + m->nout;
   a.bpart = m->bpart;
   a.rows = n;
-  wgrad_kernel<<<dim3(total, a.ks > kBiasGroups ? a.ks : kBiasGroups, m->K), kGemmThreads, kGemmSmem, s>>>(a);
+  a.members = m->K;
+  e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kWgradSmem);
+  if (e) return e;
+  const unsigned blocks = (unsigned)m->K * ((unsigned)(a.tiles[0] + a.tiles[1] + a.tiles[2]) * a.parts +
+                                            (unsigned)(a.bblocks[0] + a.bblocks[1] + a.bblocks[2]) * kBiasGroups);
+  wgrad_kernel<<<blocks, kWgradThreads, kWgradSmem, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -758,12 +1265,13 @@ static Offsets offsets(const lb_mlp* m) {
 }
 
 static cudaError_t train_step(lb_mlp* m, cudaStream_t s) {
-  cudaError_t e = backward(m, s);
+  cudaError_t e = backward(m, m->sched, s);
   if (e) return e;
   int ks, kc;
   wgrad_splits(m, m->n, &ks, &kc);
+  ks = wgrad_parts(m, ks);
   adamw_kernel<<<dim3((unsigned)((m->P / 4 + 255) / 256), m->K), 256, 0, s>>>(m->p, m->pb, m->part, m->bpart, ks, m->m1,
-                                                                           m->m2, m->P, m->sched, offsets(m));
+                                                                           m->m2, m->P, m->sched, offsets(m), m->loss);
   return cudaGetLastError();
 }
 
@@ -792,6 +1300,16 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
     return merr(NULL, "cudaStreamCreate failed"), LB_ERR_CUDA;
   }
   const long PK = m->P * members, B = max_batch;
+  int dev = 0, sms = 0, optin = 0;
+  cudaError_t ea = cudaGetDevice(&dev);
+  if (ea == cudaSuccess) ea = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (ea == cudaSuccess) ea = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (ea != cudaSuccess) {
+    lb_mlp_destroy(m);
+    return merr(NULL, "device query failed: %s", cudaGetErrorString(ea)), LB_ERR_CUDA;
+  }
+  m->sms = sms;
+  m->max_smem = (size_t)optin;
   m->p = (float*)malloc_dev(m, PK * 4);
   m->g = (float*)malloc_dev(m, PK * 4);
   m->m1 = (float*)malloc_dev(m, PK * 4);
@@ -801,6 +1319,9 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
   m->loss = (float*)malloc_dev(m, 64 * sizeof(float));
   m->xb = (bf16*)malloc_dev(m, B * 16 * 2);
   m->xbp = (bf16*)malloc_dev(m, B * 16 * 2);
+  m->xin = (float*)malloc_dev(m, B * nin * 4);
+  m->mean = (float*)malloc_dev(m, B * nout * 4);
+  m->sd = (float*)malloc_dev(m, B * nout * 4);
   m->h1 = (bf16*)malloc_dev(m, members * B * nh * 2);
   m->h2 = (bf16*)malloc_dev(m, members * B * nh * 2);
   m->dz2b = (bf16*)malloc_dev(m, members * B * nh * 2);
@@ -823,7 +1344,7 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
     m->part = (float*)malloc_dev(m, 4L * members * m->ks_max * m->P);
     m->bpart = (float*)malloc_dev(m, 4L * members * kBiasGroups * (2 * nh + nout));
   }
-  bool ok = m->part && m->bpart && m->p && m->g && m->m1 && m->m2 && m->pb && m->sched && m->loss && m->xb && m->xbp && m->h1 && m->h2 && m->dz2b &&
+  bool ok = m->part && m->bpart && m->p && m->g && m->m1 && m->m2 && m->pb && m->sched && m->loss && m->xb && m->xbp && m->xin && m->mean && m->sd && m->h1 && m->h2 && m->dz2b &&
             m->dz1b && m->dz2f && m->dz1f && m->y && m->dyf && m->dyb && m->t;
   if (!ok) {
     lb_mlp_destroy(m);
@@ -869,26 +1390,21 @@ lb_status lb_mlp_get_params(lb_mlp* m, int k, float* params) {
 
 lb_status lb_mlp_set_params(lb_mlp* m, int k, const float* params) {
   if (!m || k < 0 || k >= m->K || !params) return LB_ERR_ARG;
-  std::vector<bf16> hb(m->P);
-  for (long i = 0; i < m->P; ++i) hb[i] = __float2bfloat16(params[i]);
   MCK(cudaMemcpyAsync(m->p + k * m->P, params, m->P * 4, cudaMemcpyHostToDevice, m->stream));
-  MCK(cudaMemcpyAsync(m->pb + k * m->P, hb.data(), m->P * 2, cudaMemcpyHostToDevice, m->stream));
-  MCK(cudaMemsetAsync(m->m1 + k * m->P, 0, m->P * 4, m->stream));
-  MCK(cudaMemsetAsync(m->m2 + k * m->P, 0, m->P * 4, m->stream));
+  load_params_kernel<<<blocks_for(m, m->P / 4), 256, 0, m->stream>>>(m->p + k * m->P, m->pb + k * m->P,
+                                                                    m->m1 + k * m->P, m->m2 + k * m->P, m->P);
+  MCK(cudaGetLastError());
   MCK(cudaStreamSynchronize(m->stream));
   return LB_OK;
 }
 
 lb_status lb_mlp_set_data(lb_mlp* m, int n, const float* x, const float* y) {
   if (!m || n < 1 || n > m->maxb || !x || !y) return LB_ERR_ARG;
-  float* dx = (float*)malloc_dev(m, (size_t)n * m->nin * 4);
-  if (!dx) return merr(m, "device allocation failed"), LB_ERR_NOMEM;
-  MCK(cudaMemcpyAsync(dx, x, (size_t)n * m->nin * 4, cudaMemcpyHostToDevice, m->stream));
-  pack_x_kernel<<<64, 256, 0, m->stream>>>(dx, n, m->nin, m->xb);
+  MCK(cudaMemcpyAsync(m->xin, x, (size_t)n * m->nin * 4, cudaMemcpyHostToDevice, m->stream));
+  pack_x_kernel<<<blocks_for(m, 16L * n), 256, 0, m->stream>>>(m->xin, n, m->nin, m->xb);
   MCK(cudaGetLastError());
   MCK(cudaMemcpyAsync(m->t, y, (size_t)n * m->nout * 4, cudaMemcpyHostToDevice, m->stream));
   MCK(cudaStreamSynchronize(m->stream));
-  free_last(m);
   m->n = n;
   if (m->gexec) {
     cudaGraphExecDestroy(m->gexec);
@@ -899,9 +1415,11 @@ lb_status lb_mlp_set_data(lb_mlp* m, int n, const float* x, const float* y) {
 
 lb_status lb_mlp_gradients(lb_mlp* m, int k, float* grads, float* loss) {
   if (!m || k < 0 || k >= m->K || !grads || m->n < 1) return LB_ERR_ARG;
-  MCK(backward(m, m->stream));
+  MCK(cudaMemsetAsync(m->loss, 0, m->K * sizeof(float), m->stream));
+  MCK(backward(m, NULL, m->stream));
   int ks, kc;
   wgrad_splits(m, m->n, &ks, &kc);
+  ks = wgrad_parts(m, ks);
   grad_sum_kernel<<<256, 256, 0, m->stream>>>(m->part, m->bpart, ks, m->P, offsets(m), k, m->g);
   MCK(cudaGetLastError());
   MCK(cudaMemcpyAsync(grads, m->g + k * m->P, m->P * 4, cudaMemcpyDeviceToHost, m->stream));
@@ -914,7 +1432,7 @@ lb_status lb_mlp_gradients(lb_mlp* m, int k, float* grads, float* loss) {
 
 lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, float* losses) {
   if (!m || steps < 1 || m->n < 1 || !(lr > 0)) return LB_ERR_ARG;
-  Sched sc = {-1, steps, lr, lr_min, wd};  // every step's first kernel counts it
+  Sched sc = {-1, steps, lr, lr_min, wd};  // every step's gradient launch counts it
   MCK(cudaMemcpyAsync(m->sched, &sc, sizeof sc, cudaMemcpyHostToDevice, m->stream));
   if (!m->gexec) {
     MCK(cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeThreadLocal));
@@ -926,10 +1444,12 @@ lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, f
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) return merr(m, "graph capture failed: %s", cudaGetErrorString(e)), LB_ERR_CUDA;
   }
+  MCK(cudaMemsetAsync(m->loss, 0, m->K * sizeof(float), m->stream));
   for (int i = 0; i < steps; ++i) MCK(cudaGraphLaunch(m->gexec, m->stream));
   if (losses) {
-    // loss of the final parameters
-    MCK(forward(m, m->n, m->xb, true, m->stream));
+    // loss of the final parameters (the last update cleared the sums)
+    const int rt = rows_plan(m, m->n, true);
+    MCK(rt ? rows_train(m, rt, m->stream) : forward(m, m->n, m->xb, true, m->stream));
     MCK(cudaMemcpyAsync(losses, m->loss, m->K * 4, cudaMemcpyDeviceToHost, m->stream));
   }
   MCK(cudaStreamSynchronize(m->stream));
@@ -939,24 +1459,25 @@ lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, f
 lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* sd, float* members) {
   if (!m || n < 1 || !x || !mean || !sd) return LB_ERR_ARG;
   if (n > m->maxb) return merr(m, "batch larger than max_batch"), LB_ERR_ARG;
-  float* dx = (float*)malloc_dev(m, (size_t)n * m->nin * 4 + 2 * (size_t)n * m->nout * 4);
-  if (!dx) return merr(m, "device allocation failed"), LB_ERR_NOMEM;
-  float* dmean = dx + (size_t)n * m->nin;
-  float* dsd = dmean + (size_t)n * m->nout;
-  MCK(cudaMemcpyAsync(dx, x, (size_t)n * m->nin * 4, cudaMemcpyHostToDevice, m->stream));
-  pack_x_kernel<<<64, 256, 0, m->stream>>>(dx, n, m->nin, m->xbp);
+  MCK(cudaMemcpyAsync(m->xin, x, (size_t)n * m->nin * 4, cudaMemcpyHostToDevice, m->stream));
+  const int rt = rows_plan(m, n, false);
+  if (rt) {
+    MCK(rows_predict(m, rt, n, m->xin, m->stream));
+  } else {
+    pack_x_kernel<<<blocks_for(m, 16L * n), 256, 0, m->stream>>>(m->xin, n, m->nin, m->xbp);
+    MCK(cudaGetLastError());
+    MCK(forward(m, n, m->xbp, false, m->stream));
+  }
+  ensemble_kernel<<<blocks_for(m, (long)n * m->nout / 4), 256, 0, m->stream>>>(
+      m->y, m->K, (long)m->maxb * m->nout, (long)n * m->nout, m->mean, m->sd);
   MCK(cudaGetLastError());
-  MCK(forward(m, n, m->xbp, false, m->stream));
-  ensemble_kernel<<<64, 256, 0, m->stream>>>(m->y, m->K, (long)m->maxb * m->nout, (long)n * m->nout, dmean, dsd);
-  MCK(cudaGetLastError());
-  MCK(cudaMemcpyAsync(mean, dmean, (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
-  MCK(cudaMemcpyAsync(sd, dsd, (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
+  MCK(cudaMemcpyAsync(mean, m->mean, (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
+  MCK(cudaMemcpyAsync(sd, m->sd, (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
   if (members)
     for (int k = 0; k < m->K; ++k)
       MCK(cudaMemcpyAsync(members + (size_t)k * n * m->nout, m->y + (size_t)k * m->maxb * m->nout,
                           (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
   MCK(cudaStreamSynchronize(m->stream));
-  free_last(m);
   return LB_OK;
 }
 
