@@ -145,15 +145,16 @@ static OpArgs base_args(const lb_ctx* c) {
 }
 
 // After a synchronisation: a device-side wait that gave up poisons the context.
+static lb_status device_error(lb_ctx* c, bool failed) {
+  if (!failed) return LB_OK;
+  c->poisoned = 1;
+  set_err(c, "a device-side wait of the step kernel timed out (state is unreliable)");
+  return LB_ERR_TIMEOUT;
+}
 static lb_status check_device_error(lb_ctx* c) {
   int h = 0;
   CK(cudaMemcpy(&h, c->errflag, sizeof h, cudaMemcpyDeviceToHost));
-  if (h) {
-    c->poisoned = 1;
-    set_err(c, "a device-side wait of the step kernel timed out (state is unreliable)");
-    return LB_ERR_TIMEOUT;
-  }
-  return LB_OK;
+  return device_error(c, h != 0);
 }
 
 // A new state clears a timed-out condition: the device error word as well as the
@@ -435,7 +436,7 @@ lb_status lb_create(const lb_grid* grid, const lb_walls* walls, const lb_params*
   }
   c->nparts = kRedPartsPerSM * device_sm_count();
   c->partials = (double*)dev_alloc_owned(c, (size_t)c->nparts * RED_PARTS * sizeof(double));
-  c->red_out = (double*)dev_alloc_owned(c, 4 * sizeof(double));
+  c->red_out = (double*)dev_alloc_owned(c, 5 * sizeof(double));
   c->errflag = (int*)dev_alloc_owned(c, 256);
   if (c->errflag && cudaMemsetAsync(c->errflag, 0, 256, c->stream) != cudaSuccess) c->errflag = NULL;
   if (!c->partials || !c->red_out || !c->errflag) {
@@ -540,12 +541,11 @@ lb_status lb_filled_length(lb_ctx* c, double* l_centre, double* l_vol, double* m
   a.nparts = c->nparts;
   a.partials = c->partials;
   a.red_out = c->red_out;
-  CK(c->ops(OP_RED_PARTIALS, a, c->stream));
-  CK(c->ops(OP_RED_FINAL, a, c->stream));
-  double h[4];
+  CK(c->ops(OP_REDUCE, a, c->stream));
+  double h[5];
   CK(cudaMemcpyAsync(h, c->red_out, sizeof h, cudaMemcpyDeviceToHost, c->stream));
   CK(cudaStreamSynchronize(c->stream));
-  lb_status dst = check_device_error(c);
+  lb_status dst = device_error(c, h[4] != 0.0);
   if (dst != LB_OK) return dst;
   if (l_centre) *l_centre = h[0];
   if (l_vol) *l_vol = h[1];

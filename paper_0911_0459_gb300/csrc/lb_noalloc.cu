@@ -95,7 +95,7 @@ cudaError_t reduce(const lbk::Geom& G, const lbk::Buf<S>& B, double rho_l, doubl
   lbk::reduce_partials_kernel<MODEL, S><<<nblocks, lbk::RED_THREADS, 0, s>>>(G, B, rho_l, rho_g, thr, partials);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  lbk::reduce_final_kernel<MODEL, S><<<1, 32, 0, s>>>(G, B, thr, nblocks, partials, out);
+  lbk::reduce_final_kernel<MODEL, S><<<1, lbk::RED_FINAL_THREADS, 0, s>>>(G, B, thr, nblocks, partials, out, nullptr);
   return cudaGetLastError();
 }
 

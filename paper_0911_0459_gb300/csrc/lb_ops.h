@@ -37,7 +37,7 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-enum OpKind { OP_STEP, OP_INIT, OP_FIELDS, OP_POPS_OUT, OP_POPS_IN, OP_RED_PARTIALS, OP_RED_FINAL, OP_MOMENTS_OUT,
+enum OpKind { OP_STEP, OP_INIT, OP_FIELDS, OP_POPS_OUT, OP_POPS_IN, OP_REDUCE, OP_MOMENTS_OUT,
               OP_CHECK };
 
 struct OpBufs {
@@ -67,7 +67,7 @@ struct OpArgs {
   int flag;      // rested flag for OP_POPS_OUT
   int nparts;    // reduction partial blocks
   double* partials;
-  double* red_out;
+  double* red_out;  // {l_centre, l_vol, mass, phi_sum, device error word}
   unsigned long long* check_out;  // OP_CHECK: host array {enabled, bad accesses, first bad index + 1}
 };
 

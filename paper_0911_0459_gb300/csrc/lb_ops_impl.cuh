@@ -1,6 +1,8 @@
 // Launch wrappers of every kernel for one (model, storage) pair.
 #pragma once
 
+#include <utility>
+
 #include "lb_aux.cuh"
 #include "lb_device.cuh"
 #include "lb_ops.h"
@@ -42,12 +44,12 @@ static inline int grid_for(size_t n, int threads) {
   return (int)(b > cap ? cap : (b < 1 ? 1 : b));
 }
 
-// Launch of a step kernel that may start while the previous one on the stream
-// still runs (pdl_wait in lb_device.cuh); captured into a graph, the dependency
-// becomes a programmatic edge.
-template <class Args>
-static cudaError_t launch_pdl(void (*kernel)(Args), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
-                              const Args& k) {
+// Launch of a kernel that may start while the previous one on the stream still runs
+// (pdl_wait in lb_device.cuh); captured into a graph, the dependency becomes a
+// programmatic edge.
+template <class... P, class... A>
+static cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
+                              A&&... args) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
@@ -58,7 +60,7 @@ static cudaError_t launch_pdl(void (*kernel)(Args), unsigned grid, unsigned bloc
   cfg.stream = s;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, k);
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 template <int MODEL, class S, int BX>
@@ -157,15 +159,15 @@ cudaError_t ops_impl(OpKind op, const OpArgs& a, cudaStream_t s) {
     case OP_POPS_IN:
       pops_in_kernel<MODEL, S><<<grid_for(N, 256), 256, 0, s>>>(G, to_buf<S>(a.dst, a), a.in0, a.in1);
       return cudaGetLastError();
-    case OP_RED_PARTIALS:
-      reduce_partials_kernel<MODEL, S><<<a.nparts, RED_THREADS, 0, s>>>(G, to_buf<S>(a.src, a), a.rho_l, a.rho_g, a.thr,
-                                                                        a.partials);
-      return cudaGetLastError();
+    case OP_REDUCE: {
+      cudaError_t e = launch_pdl(reduce_partials_kernel<MODEL, S>, a.nparts, RED_THREADS, 0, s, G, to_buf<S>(a.src, a),
+                                 a.rho_l, a.rho_g, a.thr, a.partials);
+      if (e != cudaSuccess) return e;
+      return launch_pdl(reduce_final_kernel<MODEL, S>, 1, RED_FINAL_THREADS, 0, s, G, to_buf<S>(a.src, a), a.thr,
+                        a.nparts, (const double*)a.partials, a.red_out, (const int*)a.err);
+    }
     case OP_CHECK:
       return read_check_counters(a.check_out);
-    case OP_RED_FINAL:
-      reduce_final_kernel<MODEL, S><<<1, 32, 0, s>>>(G, to_buf<S>(a.src, a), a.thr, a.nparts, a.partials, a.red_out);
-      return cudaGetLastError();
   }
   return cudaErrorInvalidValue;
 }
