@@ -22,6 +22,7 @@
 
 #include "lb.h"
 #include "lb_batch.cuh"
+#include "lb_host.h"
 #include "lb_ops.h"
 
 using namespace lbk;
@@ -651,6 +652,7 @@ lb_status lb_batch_save_state(lb_batch* b, void* host, size_t bytes) {
   if (bytes != lb_batch_state_bytes(b)) return berr(b, "bytes must equal lb_batch_state_bytes"), LB_ERR_ARG;
   const int k = b->parity;
   unsigned char* h = static_cast<unsigned char*>(host);
+  populate_host(h, bytes);
   BCK(cudaMemcpyAsync(h, b->f[k], b->bytes_f, cudaMemcpyDeviceToHost, b->stream));
   if (b->bytes_g) BCK(cudaMemcpyAsync(h + b->bytes_f, b->g[k], b->bytes_g, cudaMemcpyDeviceToHost, b->stream));
   if (b->bytes_g0)
@@ -765,6 +767,7 @@ lb_status lb_batch_moments(lb_batch* b, int i, double* m) {
   OpArgs a = lattice_args(b, i, b->parity);
   a.out0 = d;
   cudaError_t e = batch_ops(b->storage)(OP_MOMENTS_OUT, a, b->stream);
+  if (e == cudaSuccess) populate_host(m, M_PLANES * N * sizeof(double));
   if (e == cudaSuccess) e = cudaMemcpyAsync(m, d, M_PLANES * N * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
   cudaError_t e2 = cudaStreamSynchronize(b->stream);
   if (b->have_alloc)
@@ -792,6 +795,8 @@ lb_status lb_batch_populations(lb_batch* b, int i, double* f, double* g, int res
   a.out0 = d;
   a.out1 = d + 9 * N;
   cudaError_t e = batch_ops(b->storage)(OP_POPS_OUT, a, b->stream);
+  const HostRange host[2] = {{f, 9 * N * sizeof(double)}, {g, 9 * N * sizeof(double)}};
+  if (e == cudaSuccess) populate_host(host, 2);
   if (e == cudaSuccess) e = cudaMemcpyAsync(f, d, 9 * N * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
   if (e == cudaSuccess && g) e = cudaMemcpyAsync(g, d + 9 * N, 9 * N * sizeof(double), cudaMemcpyDeviceToHost, b->stream);
   cudaError_t e2 = cudaStreamSynchronize(b->stream);

@@ -13,6 +13,7 @@
 
 #include "lb.h"
 #include "lb_aux.cuh"
+#include "lb_host.h"
 #include "lb_ops.h"
 
 using namespace lbk;
@@ -521,6 +522,9 @@ lb_status lb_fields(lb_ctx* c, double* rho, double* ux, double* uy, double* phi)
   lb_status st = LB_OK;
   cudaError_t e = c->ops(OP_FIELDS, a, c->stream);
   double* dst[4] = {rho, ux, uy, phi};
+  const HostRange host[4] = {{rho, N * sizeof(double)}, {ux, N * sizeof(double)}, {uy, N * sizeof(double)},
+                             {phi, N * sizeof(double)}};
+  if (e == cudaSuccess) populate_host(host, 4);  // beside the kernels that are still running
   for (int k = 0; k < 4 && e == cudaSuccess; ++k)
     if (dst[k]) e = cudaMemcpyAsync(dst[k], d + k * N, N * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   cudaError_t e2 = cudaStreamSynchronize(c->stream);
@@ -573,6 +577,8 @@ lb_status lb_get_populations(lb_ctx* c, double* f, double* g, int rested) {
   a.out0 = d;
   a.out1 = bin ? d + 9 * N : NULL;
   cudaError_t e = c->ops(OP_POPS_OUT, a, c->stream);
+  const HostRange host[2] = {{f, 9 * N * sizeof(double)}, {bin ? g : NULL, 9 * N * sizeof(double)}};
+  if (e == cudaSuccess) populate_host(host, 2);
   if (e == cudaSuccess) e = cudaMemcpyAsync(f, d, 9 * N * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   if (e == cudaSuccess && bin && g)
     e = cudaMemcpyAsync(g, d + 9 * N, 9 * N * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
@@ -622,6 +628,7 @@ lb_status lb_save_state(lb_ctx* c, void* host, size_t bytes) {
   if (bytes != total) return set_err(c, "bytes must equal lb_state_bytes (%zu)", total), LB_ERR_ARG;
   const OpBufs& b = c->buf[c->cur];
   unsigned char* h = static_cast<unsigned char*>(host);
+  populate_host(h, total);
   CK(cudaMemcpyAsync(h, b.f, fb, cudaMemcpyDeviceToHost, c->stream));
   if (gb) CK(cudaMemcpyAsync(h + fb, b.g, gb, cudaMemcpyDeviceToHost, c->stream));
   if (g0b) CK(cudaMemcpyAsync(h + fb + gb, b.g0, g0b, cudaMemcpyDeviceToHost, c->stream));
@@ -656,6 +663,7 @@ lb_status lb_get_moments(lb_ctx* c, double* m) {
   a.src = c->buf[c->cur];
   a.out0 = d;
   cudaError_t e = c->ops(OP_MOMENTS_OUT, a, c->stream);
+  if (e == cudaSuccess) populate_host(m, (size_t)M_PLANES * N * sizeof(double));
   if (e == cudaSuccess) e = cudaMemcpyAsync(m, d, (size_t)M_PLANES * N * sizeof(double), cudaMemcpyDeviceToHost, c->stream);
   cudaError_t e2 = cudaStreamSynchronize(c->stream);
   if (e == cudaSuccess) e = e2;

@@ -26,6 +26,7 @@
 #include <new>
 #include <vector>
 
+#include "lb_host.h"
 #include "lb_mlp.h"
 
 namespace {
@@ -1471,6 +1472,9 @@ lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* s
   ensemble_kernel<<<blocks_for(m, (long)n * m->nout / 4), 256, 0, m->stream>>>(
       m->y, m->K, (long)m->maxb * m->nout, (long)n * m->nout, m->mean, m->sd);
   MCK(cudaGetLastError());
+  const size_t out = (size_t)n * m->nout * 4;
+  const lbk::HostRange host[3] = {{mean, out}, {sd, out}, {members, out * m->K}};
+  lbk::populate_host(host, 3);  // beside the kernels
   MCK(cudaMemcpyAsync(mean, m->mean, (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
   MCK(cudaMemcpyAsync(sd, m->sd, (size_t)n * m->nout * 4, cudaMemcpyDeviceToHost, m->stream));
   if (members)
