@@ -161,18 +161,22 @@ __device__ __forceinline__ bool grid_barrier_checked(GridBarrier* b, unsigned in
 // finish the previous tile.  Every lattice's nx is a multiple of 8 (the copies'
 // 16-byte alignment).  Per-node arithmetic is the single-lattice kernels', so
 // results are bitwise those of lb_step with the staged kernel.
-// Resident CTAs per SM of the staged batch body: those of the single-lattice
-// kernel, except that the FP16 block storage keeps 80 registers per thread (its
-// batch body, which also walks the tile list, spilled at 72: 46.4 instead of
-// 43.6 GLUPS on the 256-capillary sweep with one CTA fewer per SM).
+// Resident CTAs per SM of the staged batch body: those of the single-lattice kernel for
+// the planar storages, whose copies set the pace, and few enough for the block storages
+// that nothing spills.  The batch body, which walks the tile list and holds the code for
+// rows on and off block boundaries, needs more registers than the single-lattice kernel;
+// compiled for the CTAs that shared memory holds it spilled 160 bytes a thread, which
+// cost more than the warps brought (256-capillary sweep, 128 x 16 tiles, GLUPS: FP32
+// blocks 28.8 at four CTAs, 37.1 at three, 37.2 at two; FP16 blocks 31.0 at five, 40.5,
+// 44.2 and 38.8 at four, three and two; at 64 columns 20.7 and 25.3 at six, 29.9 and
+// 34.5 at four; at 256 columns 32.3 and 46.2 at three, 34.9 and 46.2 at two).
 template <class S, int BX, int NS>
 constexpr int batch_min_blocks() {
-  if constexpr (std::is_same<S, SF16B>::value) {
+  if constexpr (is_blocked<S>::value) {
     using L = TmaLayout<MODEL_BINARY, S, BX, NS>;
     constexpr int by_smem = int(233472 / (L::BYTES + 1024));
-    constexpr int by_regs = 65536 / ((BX + 32) * 80);
-    constexpr int b = by_smem < by_regs ? by_smem : by_regs;
-    return b < 1 ? 1 : (b > 8 ? 8 : b);
+    constexpr int by_regs = BX == 64 ? 4 : (BX == 128 ? 3 : 2);
+    return by_smem < by_regs ? (by_smem < 1 ? 1 : by_smem) : by_regs;
   } else {
     return tma_min_blocks_of<MODEL_BINARY, S, BX, NS>();
   }
