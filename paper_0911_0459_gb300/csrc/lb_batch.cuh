@@ -162,21 +162,25 @@ __device__ __forceinline__ bool grid_barrier_checked(GridBarrier* b, unsigned in
 // 16-byte alignment).  Per-node arithmetic is the single-lattice kernels', so
 // results are bitwise those of lb_step with the staged kernel.
 // Resident CTAs per SM of the staged batch body: those of the single-lattice kernel for
-// the planar storages, whose copies set the pace, and few enough for the block storages
-// that nothing spills.  The batch body, which walks the tile list and holds the code for
-// rows on and off block boundaries, needs more registers than the single-lattice kernel;
-// compiled for the CTAs that shared memory holds it spilled 160 bytes a thread, which
-// cost more than the warps brought (256-capillary sweep, 128 x 16 tiles, GLUPS: FP32
-// blocks 28.8 at four CTAs, 37.1 at three, 37.2 at two; FP16 blocks 31.0 at five, 40.5,
-// 44.2 and 38.8 at four, three and two; at 64 columns 20.7 and 25.3 at six, 29.9 and
-// 34.5 at four; at 256 columns 32.3 and 46.2 at three, 34.9 and 46.2 at two).
+// the planar storages, whose copies set the pace, and few for the block storages.  The
+// batch body, which walks the tile list and holds the code for rows on and off block
+// boundaries, needs more registers than the single-lattice kernel; compiled for the CTAs
+// that shared memory holds it spilled 160 bytes a thread, which cost more than the warps
+// brought.  Beyond that the FP32 blocks, which HBM bounds, run faster with fewer rows in
+// flight at a time, while the FP16 blocks, which instructions bound, want their warps
+// (256-capillary sweep, bands of 16 rows, GLUPS):
+//   FP32 blocks  128 columns: 28.8, 36.6, 38.7 at 4, 3, 2 CTAs;  64: 20.7, 31.4, 34.8 at
+//                6, 5, 4 (3: 34.8);  256: 34.7, 36.9 (deep ring) at 2, 1
+//   FP16 blocks  128 columns: 31.0, 46.5, 40.3 at 5, 3, 2 CTAs;  64: 25.3, 32.5, 35.4 at
+//                6, 5, 4 (3: 35.2);  256: 46.2, 49.0, 38.4 at 3, 2, 1
 template <class S, int BX, int NS>
 constexpr int batch_min_blocks() {
   if constexpr (is_blocked<S>::value) {
     using L = TmaLayout<MODEL_BINARY, S, BX, NS>;
+    constexpr bool F16 = std::is_same<S, SF16B>::value;
     constexpr int by_smem = int(233472 / (L::BYTES + 1024));
-    constexpr int by_regs = BX == 64 ? 4 : (BX == 128 ? 3 : 2);
-    return by_smem < by_regs ? (by_smem < 1 ? 1 : by_smem) : by_regs;
+    constexpr int few = BX == 64 ? 4 : (BX == 128 ? (F16 ? 3 : 2) : (F16 ? 2 : 1));
+    return by_smem < few ? (by_smem < 1 ? 1 : by_smem) : few;
   } else {
     return tma_min_blocks_of<MODEL_BINARY, S, BX, NS>();
   }

@@ -402,6 +402,41 @@ __device__ __forceinline__ void push_node_blk16(__half* __restrict__ f, float* _
   }
 }
 
+// The same pairs when rows start inside blocks (nx % 32 != 0): a node's address takes
+// three operations, with 32 b = n - n % 32 (B floats or halves per block, the pairs 2 wide)
+// B (n / 32) + 2 (n % 32) = (B / 32) n - (B / 32 - 2) (n % 32).
+template <int MODEL, class S>
+__device__ __forceinline__ void push_node_blk_rows(const Buf<S>& dst, unsigned long long lim, const int rowb[3],
+                                                   const int col[3], const bool sol[3][3], bool bnd,
+                                                   const float fs[9], const float ge[9]) {
+  static_assert(MODEL == MODEL_BINARY, "the block storages hold the binary model");
+  constexpr bool F32 = std::is_same<S, SF32B>::value;
+  constexpr uint32_t K = S::kBlock / 32;
+  const uint32_t self = (uint32_t)(rowb[1] + col[1]);
+  if constexpr (!F32) {
+    const uint32_t r = self & 31u;
+    LB_GUARD(K * self - (K - 1) * r, lim, );
+    dst.f[K * self - (K - 1) * r] = __float2half_rn(fs[0]);
+    LB_GUARD((self >> 5) * SF16B::kG0Stride + r, lim / 2 - SF16B::kG0, );
+    dst.g0[(self >> 5) * SF16B::kG0Stride + r] = ge[0];
+  }
+#pragma unroll
+  for (int i = F32 ? 0 : 1; i < 9; ++i) {
+    const int ex = EXd(i), ey = EYd(i);
+    const bool back = bnd && sol[1 + ey][1 + ex];
+    const uint32_t n = back ? self : (uint32_t)(rowb[1 + ey] + col[1 + ex]);
+    const int di = back ? OPPd(i) : i;
+    const uint32_t base = K * n - (K - 2) * (n & 31u);
+    if constexpr (F32) {
+      LB_GUARD((unsigned long long)base + 64 * di + 1, lim, );
+      *reinterpret_cast<float2*>(dst.f + base + 64 * di) = make_float2(fs[i], ge[i]);
+    } else {
+      LB_GUARD((unsigned long long)base + 32 + 64 * (di - 1) + 1, lim, );
+      *reinterpret_cast<__half2*>(dst.f + base + 32 + 64 * (di - 1)) = __floats2half2_rn(fs[i], ge[i]);
+    }
+  }
+}
+
 // UROWS: block storage with rows that start inside a block (nx % 32 != 0): the
 // stage columns of a lane change from row to row (a separate instantiation, so
 // that aligned rows keep constant columns and no per-row work).
@@ -550,7 +585,7 @@ __device__ bool consume_tile(const Ring<MODEL, S, BX, NS>& R, const Geom& G, con
   // band are solid throughout
   const bool warp_all_tube = __all_sync(0xffffffffu, tc[0] && tc[1] && tc[2]);
   auto solid_row = [&](int y) { return warp_all_tube && !row_in_band(G, wrapi(y, ny)); };
-  const uint32_t N32 = (uint32_t)N;
+  [[maybe_unused]] const uint32_t N32 = (uint32_t)N;
   // block storage, rows on block boundaries: the column parts of this lane's three
   // destination columns' block addresses
   constexpr bool BA = L::BLK && !UROWS;
@@ -558,11 +593,11 @@ __device__ bool consume_tile(const Ring<MODEL, S, BX, NS>& R, const Geom& G, con
   [[maybe_unused]] uint32_t cpart_f0 = 0u;  // SF16B: this lane's f_0 half, less its row's part
   [[maybe_unused]] uint32_t cpart_g0 = 0u;  // SF16B: this lane's g_0 float, less its row's part
   [[maybe_unused]] unsigned long long blk_lim = 0;
+  if constexpr (L::BLK) blk_lim = (unsigned long long)(N + 31) / 32 * S::kBlock;
   if constexpr (BA) {
     constexpr int B = S::kBlock;
 #pragma unroll
     for (int i = 0; i < 3; ++i) cpart[i] = (uint32_t)(col[i] >> 5) * B + 2u * (uint32_t)(col[i] & 31);
-    blk_lim = (unsigned long long)(N + 31) / 32 * B;
     if constexpr (!std::is_same<S, SF32B>::value) {
       cpart_f0 = (uint32_t)(x >> 5) * B + (uint32_t)(x & 31);
       cpart_g0 = (uint32_t)(x >> 5) * SF16B::kG0Stride + (uint32_t)(x & 31);
@@ -578,6 +613,8 @@ __device__ bool consume_tile(const Ring<MODEL, S, BX, NS>& R, const Geom& G, con
       else
         push_node_blk16<MODEL>(dst.f, dst.g0, blk_lim, rpart, cpart, rpart[1] + cpart_f0,
                                (uint32_t)(rowb[1] >> 5) * SF16B::kG0Stride + cpart_g0, sol, bnd, fs, ge);
+    } else if constexpr (L::BLK) {
+      push_node_blk_rows<MODEL, S>(dst, blk_lim, rowb, col, sol, bnd, fs, ge);
     } else {
       push_node_u32<MODEL, S, RAW>(dst, N32, rowb, col, sol, bnd, fs, ge);
     }
