@@ -270,9 +270,9 @@ long lb_fluid_nodes(const lb_ctx *ctx);
 lb_status lb_set_tile(lb_ctx *ctx, int tile_x, int tile_y);
 lb_status lb_get_tile(const lb_ctx *ctx, int *tile_x, int *tile_y);
 
-/* Choose the step kernel: 0 = automatic (the staged kernel whenever it fits,
- * else the sliding-window kernel), 1 = sliding-window kernel (rows held in
- * registers), 2 = staged kernel (rows brought into shared memory by bulk
+/* Choose the step kernel: 0 = automatic (the staged kernel where it fits and the
+ * lattice is not small, else the sliding-window kernel), 1 = sliding-window kernel
+ * (rows held in registers), 2 = staged kernel (rows brought into shared memory by bulk
  * copies; fits when nx % 8 == 0 and nx * ny <= 477218588, and at any nx for
  * the block storages, else LB_ERR_ARG)
  * with its shallow ring of row stages, 3 = staged kernel with its deep ring.

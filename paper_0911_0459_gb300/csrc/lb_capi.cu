@@ -121,6 +121,25 @@ static bool staged_ok(int storage, int nx, int ny) {
   return storage == LB_STORAGE_F32_BLOCKED || storage == LB_STORAGE_F16_BLOCKED || staged_fits(nx, ny);
 }
 
+// The automatic kernel: staged where it fits, except on small lattices, where the warp
+// strips of the sliding-window variant have the shorter chain of latencies.  The planar
+// storages' rings (18 copies a row) take longest to fill; us per step, staged -> strips:
+// 704 x 40 FP32 6.1 -> 2.8, 2048 x 64 7.4 -> 5.7, 1000 x 200 9.6 -> 7.8, 4096 x 128 14.6 ->
+// 15.0; liquid-gas FP64 256 x 32 9.0 -> 7.0, 1000 x 200 61.6 -> 55.2, 4096 x 128 118 -> 122;
+// binary FP64 1024 x 64 37.3 -> 34.7, 2048 x 64 52.9 -> 62.1; FP32 blocks (one copy a row)
+// 704 x 40 3.2 -> 2.9, 1024 x 64 4.1 -> 4.1.
+static bool auto_staged(const lb_ctx* c) {
+  if (!staged_ok(c->prm.storage, c->grid.nx, c->grid.ny)) return false;
+  long strips;  // largest number of fluid nodes that runs as strips
+  switch (c->prm.storage) {
+    case LB_STORAGE_F64: strips = c->prm.model == LB_MODEL_LIQUID_GAS ? 250000 : 70000; break;
+    case LB_STORAGE_F32_BLOCKED: strips = 40000; break;
+    case LB_STORAGE_F16_BLOCKED: strips = 0; break;
+    default: strips = 300000;
+  }
+  return c->fluid > strips;
+}
+
 static OpArgs base_args(const lb_ctx* c) {
   OpArgs a;
   memset(&a, 0, sizeof a);
@@ -139,7 +158,7 @@ static OpArgs base_args(const lb_ctx* c) {
   a.thr = p.model == LB_MODEL_LIQUID_GAS ? 0.5 * (p.rho_l + p.rho_g) : 0.0;
   a.bx = c->tile_x;
   a.yc = c->tile_y;
-  a.staged = c->kernel == 2 || (c->kernel == 0 && staged_ok(c->prm.storage, c->grid.nx, c->grid.ny));
+  a.staged = c->kernel == 2 || (c->kernel == 0 && auto_staged(c));
   a.deep = c->deep;
   a.err = c->errflag;
   return a;
@@ -328,25 +347,38 @@ static lb_status default_state(lb_ctx* c) {
 // SMs idle (256 x 32 FP64 at 128 x 16 is four CTAs); bands of one row recompute the
 // sums of two halo rows for each row, which no longer pays once a wave is full.
 // Measured in us per step, 128 x 16 for every lattice against this rule:
-//   256 x 32 liquid-gas FP64      84.0   9.0 (64 x 1)
-//   700 x 40 FP32 planes          15.8   3.5 (128 x 1)
-//   2048 x 64 FP32 planes         27.1   7.4 (256 x 1)      FP32 blocks  13.6   5.5 (128 x 2)
+//   256 x 32 liquid-gas FP64      84.0   7.0 (64 x 1)
+//   700 x 40 FP32 planes          15.8   2.8 (64 x 1)
+//   2048 x 64 FP32 planes         27.1   5.7 (64 x 2)       FP32 blocks  13.6   5.5 (128 x 2)
 //   4096 x 128 FP32 blocks        17.6  11.2 (128 x 6)      moments      15.0  11.3 (128 x 6)
 //   16384 x 256 FP32 blocks       85.4  79.6 (128 x 8)      moments      50.5  48.2 (128 x 12)
 //   16384 x 256 FP32 planes       97.0  90.5 (256 x 8)      FP64         888   838 (64 x 10)
 static void default_tile(lb_ctx* c) {
   const int nx = c->grid.nx, ny = c->grid.ny, st = c->prm.storage;
   const bool lg = c->prm.model == LB_MODEL_LIQUID_GAS;
-  int bx = 128, cols = 128, per_sm, most;  // CTAs per SM in one wave; tallest band
+  int bx = 128, cols = 128, most;  // tallest band
+  double per_sm;                   // CTAs per SM in one wave
   if (pull_storage(st)) {
     // 30 columns a warp; a band also collides the two rows beside it, so taller bands
     // on two thirds of the seven resident CTAs
     cols = 120;
-    per_sm = 4;
+    per_sm = 14.0 / 3.0;
     most = 12;
-  } else if (!staged_ok(st, nx, ny)) {  // sliding window
-    per_sm = 4;
-    most = 16;
+  } else if (!auto_staged(c)) {
+    // warp strips of 30 columns, about 15 of them resident on an SM: one row each while
+    // that fills one wave at most, else up to four rows, eight on the largest lattices
+    // (4097 x 128 FP32: 15.1, 16.0 us at 4, 8 rows; 16391 x 256: 103.8, 101.3 us)
+    const double strips = (double)((nx + 29) / 30) * ((double)c->fluid / nx), wave = 15.0 * device_sm_count();
+    const bool f64 = st == LB_STORAGE_F64, small = staged_ok(st, nx, ny) || strips <= 2 * wave;
+    if (!f64 || small) {
+      const double y = ceil(strips / wave);
+      c->tile_x = 64;
+      c->tile_y = f64 ? (y < 2 ? 1 : 2) : (y <= 4 ? (y < 1 ? 1 : (int)y) : (strips > 16 * wave ? 8 : 4));
+      if (c->tile_y > ny) c->tile_y = ny;
+      return;
+    }
+    per_sm = 4;  // FP64 at a width the staged kernel does not take: the shared window
+    most = 24;
   } else if (st == LB_STORAGE_F32_BLOCKED) {
     per_sm = 4;
     most = 8;
@@ -373,7 +405,7 @@ static void default_tile(lb_ctx* c) {
   }
   // rows of column blocks, less the solid share
   const double rows = (double)((nx + cols - 1) / cols) * ((double)c->fluid / nx);
-  const double y = ceil(rows / ((double)per_sm * device_sm_count()));
+  const double y = ceil(rows / (per_sm * device_sm_count()));
   c->tile_x = bx;
   c->tile_y = y < most ? (y < 1 ? 1 : (int)y) : most;
   if (c->tile_y > ny) c->tile_y = ny;
@@ -705,7 +737,7 @@ lb_status lb_get_kernel(const lb_ctx* c, int* variant) {
     *variant = 4;
     return LB_OK;
   }
-  const int k = c->kernel == 0 ? (staged_ok(c->prm.storage, c->grid.nx, c->grid.ny) ? 2 : 1) : c->kernel;
+  const int k = c->kernel == 0 ? (auto_staged(c) ? 2 : 1) : c->kernel;
   *variant = k == 2 && c->deep ? 3 : k;
   return LB_OK;
 }

@@ -1213,6 +1213,128 @@ __device__ __forceinline__ void step_band(const Geom& G, const Phys<typename S::
   }
 }
 
+// The same update with no shared memory and no barrier: a warp owns 30 columns of the band
+// (32 lanes, of which the outer two only supply the neighbours) and takes the
+// neighbouring columns by shuffles; the loads of the rows y0 - 1 .. y0 + 1 are all issued
+// before the first sum.  A lattice of one wave is bound by the chain of latencies of a
+// step (launch, loads, sums, collision, stores), which the window's halo columns (a second
+// load and sum by two lanes of a warp) and barriers lengthen; on lattices of many waves
+// the two idle lanes cost less than the barriers in FP32.  Us per step, shared window ->
+// strips, best tile of each: 704 x 40 FP32 planes 3.68 -> 2.76, 2048 x 64 6.43 -> 5.58,
+// 1000 x 200 8.14 -> 7.79, 16391 x 256 104.4 -> 101.3; 256 x 32 liquid-gas FP64 8.5 ->
+// 7.0 (its FP64 sums without the halo columns).
+constexpr int kStripCols = 30;
+
+template <int MODEL, class S>
+__device__ __forceinline__ void step_strip(const Geom& G, const Phys<typename S::A>& P, const MomPhys& Q,
+                                           const Buf<S>& src, const Buf<S>& dst, int c0, int y0, int y1) {
+  using A = typename S::A;
+  constexpr bool BIN = MODEL == MODEL_BINARY;
+  constexpr bool RAW = dev_arith<S>::value;
+  constexpr unsigned FULL = 0xffffffffu;
+  const int nx = G.nx, ny = G.ny;
+  const size_t N = (size_t)nx * ny;
+  const int lane = threadIdx.x & 31;
+  const int c = c0 - 1 + lane;  // this lane's column, -1 .. nx standing for the wrapped ones
+  const int x = c < 0 ? nx - 1 : (c < nx ? c : (c - nx < nx ? c - nx : 0));
+  const bool act = lane > 0 && lane <= kStripCols && c < nx;
+  const int xm = x == 0 ? nx - 1 : x - 1, xp = x + 1 >= nx ? 0 : x + 1;
+  const bool tubed = G.tube_len > 0;
+  const bool tc[3] = {tubed && col_in_tube(G, xm), tubed && col_in_tube(G, x), tubed && col_in_tube(G, xp)};
+  struct Row {
+    A rc, rl, rr, pc, pl, pr;
+  };
+  auto load = [&](int r, A* f, A* g) {
+    const int rr = wrapi(r, ny);
+    const bool fluid = !(tc[1] && !row_in_band(G, rr));
+    if (fluid) load_node<MODEL, S, false, RAW>(src, N, (size_t)rr * nx + x, f, g);
+    return fluid;
+  };
+  auto sums = [&](const A* f, const A* g, bool fluid) {
+    Row w;
+    w.rc = fluid ? sum9(f) : A(0);
+    w.rl = __shfl_up_sync(FULL, w.rc, 1);
+    w.rr = __shfl_down_sync(FULL, w.rc, 1);
+    w.pc = w.pl = w.pr = A(0);
+    if (BIN) {
+      w.pc = fluid ? sum9(g) : A(0);
+      w.pl = __shfl_up_sync(FULL, w.pc, 1);
+      w.pr = __shfl_down_sync(FULL, w.pc, 1);
+    }
+    return w;
+  };
+  A fa[9], fb[9], fc[9], g0[9], g1[9], g2[9];
+  bool fl_a, fl_b, fl_c;
+  Row Rw[3];
+  {
+    fl_c = load(y0 - 1, fc, g0);
+    fl_a = load(y0, fa, g1);
+    fl_b = load(y0 + 1, fb, g2);
+    Rw[0] = sums(fc, g0, fl_c);
+    Rw[1] = sums(fa, g1, fl_a);
+    Rw[2] = sums(fb, g2, fl_b);
+  }
+  for (int y = y0; y < y1; ++y) {
+    const bool more = y + 1 < y1;
+    if (more) fl_c = load(y + 2, fc, g0);
+    if (act && fl_a) {
+      const int yy = wrapi(y, ny);
+      const int ym = yy == 0 ? ny - 1 : yy - 1, yp = yy + 1 >= ny ? 0 : yy + 1;
+      const bool rb[3] = {row_in_band(G, ym), row_in_band(G, yy), row_in_band(G, yp)};
+      bool sol[3][3], bnd = false;
+      A vr[3][3], vp[3][3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          sol[j][i] = tc[i] && !rb[j];
+          bnd = bnd || sol[j][i];
+        }
+        vr[j][0] = Rw[j].rl;
+        vr[j][1] = Rw[j].rc;
+        vr[j][2] = Rw[j].rr;
+        if (BIN) {
+          vp[j][0] = Rw[j].pl;
+          vp[j][1] = Rw[j].pc;
+          vp[j][2] = Rw[j].pr;
+        }
+      }
+      A fs[9], ge[9];
+      if constexpr (RAW)
+        collide_node_f16<MODEL>(Q, vr, vp, sol, bnd, fa, fs, ge);
+      else
+        collide_node<MODEL, A>(P, vr, vp, sol, bnd, fa, fs, ge);
+      const int rowb[3] = {ym * nx, yy * nx, yp * nx};
+      const int col[3] = {xm, x, xp};
+      push_node<MODEL, S, RAW>(dst, N, rowb, col, sol, bnd, fs, ge);
+    }
+    if (more) {
+      Rw[0] = Rw[1];
+      Rw[1] = Rw[2];
+      Rw[2] = sums(fc, g0, fl_c);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        fa[i] = fb[i];
+        fb[i] = fc[i];
+      }
+      fl_a = fl_b;
+      fl_b = fl_c;
+    }
+  }
+}
+
+template <int MODEL, class S, int NW>
+__global__ void __launch_bounds__(NW * 32) strip_kernel(StepArgs<MODEL, S> a) {
+  int cb, band;
+  tile_of_block((a.G.nx + NW * kStripCols - 1) / (NW * kStripCols), cb, band);
+  const int c0 = (cb * NW + (int)(threadIdx.x >> 5)) * kStripCols;
+  const int y0 = band * a.yc;
+  const int y1 = min(y0 + a.yc, a.G.ny);
+  pdl_wait();
+  if (c0 < a.G.nx) step_strip<MODEL, S>(a.G, a.P, a.Q, a.src, a.dst, c0, y0, y1);
+  pdl_trigger();
+}
+
 template <int MODEL, class S, int BX>
 __global__ void __launch_bounds__(BX) step_kernel(StepArgs<MODEL, S> a) {
   __shared__ StepSmem<MODEL, S, BX> sm;

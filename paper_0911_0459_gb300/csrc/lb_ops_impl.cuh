@@ -63,6 +63,13 @@ static cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned bloc
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// The sliding-window variant runs as warp strips (step_strip).  In FP64 only bands of one
+// or two rows do: there the FP64 pipe is the bound and the strips' 32 lanes for 30 columns
+// cost more than the window's barriers on lattices that fill the GPU (liquid-gas, us per
+// step: 256 x 32 at one row 8.5 -> 7.0, 4097 x 128 at two rows 123.1 -> 122.3, at six
+// 118.4 -> 127.6).
+constexpr int kStripRowsF64 = 2;
+
 template <int MODEL, class S, int BX>
 static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
   StepArgs<MODEL, S> k;
@@ -72,8 +79,12 @@ static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
   k.src = to_buf<S>(a.src, a);
   k.dst = to_buf<S>(a.dst, a);
   k.yc = a.yc;
-  const unsigned grid = tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc);
-  return launch_pdl(step_kernel<MODEL, S, BX>, grid, BX, 0, s, k);
+  if constexpr (std::is_same<typename S::A, double>::value) {
+    if (a.yc > kStripRowsF64)
+      return launch_pdl(step_kernel<MODEL, S, BX>, tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc), BX, 0, s, k);
+  }
+  return launch_pdl(strip_kernel<MODEL, S, BX / 32>,
+                    tiles_1d((a.nx + BX / 32 * kStripCols - 1) / (BX / 32 * kStripCols), a.ny, a.yc), BX, 0, s, k);
 }
 
 template <int MODEL, class S, int BX, int NS>
