@@ -127,17 +127,19 @@ static bool staged_ok(int storage, int nx, int ny) {
 // 704 x 40 FP32 6.1 -> 2.8, 2048 x 64 7.4 -> 5.7, 1000 x 200 9.6 -> 7.8, 4096 x 128 14.6 ->
 // 15.0; liquid-gas FP64 256 x 32 9.0 -> 7.0, 1000 x 200 61.6 -> 55.2, 4096 x 128 118 -> 122;
 // binary FP64 1024 x 64 37.3 -> 34.7, 2048 x 64 52.9 -> 62.1; FP32 blocks (one copy a row)
-// 704 x 40 3.2 -> 2.9, 1024 x 64 4.1 -> 4.1.
+// 704 x 40 3.2 -> 2.6, 1024 x 64 4.2 -> 3.5, 2048 x 64 5.6 -> 5.3, 1000 x 200 7.2 -> 7.1, 4096 x
+// 128 11.2 -> 13.8; FP16 blocks 704 x 40 3.2 -> 3.4, 1024 x 64 4.2 -> 3.7, 2048 x 64 5.5 -> 5.3,
+// 1000 x 200 6.7 -> 7.2.
 static bool auto_staged(const lb_ctx* c) {
   if (!staged_ok(c->prm.storage, c->grid.nx, c->grid.ny)) return false;
-  long strips;  // largest number of fluid nodes that runs as strips
+  long strips, least = 0;  // largest and smallest number of fluid nodes that runs as strips
   switch (c->prm.storage) {
     case LB_STORAGE_F64: strips = c->prm.model == LB_MODEL_LIQUID_GAS ? 250000 : 70000; break;
-    case LB_STORAGE_F32_BLOCKED: strips = 40000; break;
-    case LB_STORAGE_F16_BLOCKED: strips = 0; break;
+    case LB_STORAGE_F32_BLOCKED: strips = 150000; break;
+    case LB_STORAGE_F16_BLOCKED: strips = 120000, least = 40000; break;
     default: strips = 300000;
   }
-  return c->fluid > strips;
+  return c->fluid > strips || c->fluid < least;
 }
 
 static OpArgs base_args(const lb_ctx* c) {
@@ -349,7 +351,7 @@ static lb_status default_state(lb_ctx* c) {
 // Measured in us per step, 128 x 16 for every lattice against this rule:
 //   256 x 32 liquid-gas FP64      84.0   7.0 (64 x 1)
 //   700 x 40 FP32 planes          15.8   2.8 (64 x 1)
-//   2048 x 64 FP32 planes         27.1   5.7 (64 x 2)       FP32 blocks  13.6   5.5 (128 x 2)
+//   2048 x 64 FP32 planes         27.1   5.7 (64 x 2)       FP32 blocks  13.6   5.3 (64 x 2)
 //   4096 x 128 FP32 blocks        17.6  11.2 (128 x 6)      moments      15.0  11.3 (128 x 6)
 //   16384 x 256 FP32 blocks       85.4  79.6 (128 x 8)      moments      50.5  48.2 (128 x 12)
 //   16384 x 256 FP32 planes       97.0  90.5 (256 x 8)      FP64         888   838 (64 x 10)

@@ -304,6 +304,14 @@ struct SF32B {
     fv = v.x;
     gv = v.y;
   }
+  // the same from global memory (f: the buffer's f base)
+  __device__ static void lfg(const T* __restrict__ f, const float*, size_t N, size_t n, int i, A& fv, A& gv) {
+    fv = gv = A(0);
+    LB_GUARD(at(n, i) + 1, lim(N), );
+    const float2 v = __ldg(reinterpret_cast<const float2*>(f + at(n, i)));
+    fv = v.x;
+    gv = v.y;
+  }
   __device__ static A lf(const T* __restrict__ f, size_t N, size_t n, int i, const Rest&) {
     LB_GUARD(at(n, i), lim(N), A(0));
     return __ldg(f + at(n, i));
@@ -379,6 +387,20 @@ struct SF16B {
   // stage's f base)
   __device__ static void pfg(const T* f, const float*, int c, int i, A& fv, A& gv) {
     const float2 v = __half22float2(*reinterpret_cast<const __half2*>(f + sat(c, i)));
+    fv = v.x;
+    gv = v.y;
+  }
+  // the same from global memory; i = 0: f_0 - w_0 and the FP32 g_0
+  __device__ static void lfg(const T* __restrict__ f, const float* __restrict__ g0, size_t N, size_t n, int i, A& fv,
+                             A& gv) {
+    fv = gv = 0.0f;
+    if (i == 0) {
+      fv = lfr(f, N, n, 0);
+      gv = lg(f + kGOff, g0, N, n, 0);
+      return;
+    }
+    LB_GUARD(at(n, i) + 1, lim(N), );
+    const float2 v = __half22float2(__ldg(reinterpret_cast<const __half2*>(f + at(n, i))));
     fv = v.x;
     gv = v.y;
   }
@@ -1080,6 +1102,41 @@ __device__ __forceinline__ void push_node_u32(const Buf<S>& dst, uint32_t N, con
   }
 }
 
+// push_node for the block storages at any width, each pair (f_i, g_i) as one store: a
+// node's address takes three operations (B floats or halves per block, the pairs 2 wide):
+// B (n / 32) + 2 (n % 32) = (B / 32) n - (B / 32 - 2) (n % 32).  lim: elements of the state.
+template <int MODEL, class S>
+__device__ __forceinline__ void push_node_blk_rows(const Buf<S>& dst, unsigned long long lim, const int rowb[3],
+                                                   const int col[3], const bool sol[3][3], bool bnd,
+                                                   const float fs[9], const float ge[9]) {
+  static_assert(MODEL == MODEL_BINARY, "the block storages hold the binary model");
+  constexpr bool F32 = std::is_same<S, SF32B>::value;
+  constexpr uint32_t K = S::kBlock / 32;
+  const uint32_t self = (uint32_t)(rowb[1] + col[1]);
+  if constexpr (!F32) {
+    const uint32_t r = self & 31u;
+    LB_GUARD(K * self - (K - 1) * r, lim, );
+    dst.f[K * self - (K - 1) * r] = __float2half_rn(fs[0]);
+    LB_GUARD((self >> 5) * SF16B::kG0Stride + r, lim / 2 - SF16B::kG0, );
+    dst.g0[(self >> 5) * SF16B::kG0Stride + r] = ge[0];
+  }
+#pragma unroll
+  for (int i = F32 ? 0 : 1; i < 9; ++i) {
+    const int ex = EXd(i), ey = EYd(i);
+    const bool back = bnd && sol[1 + ey][1 + ex];
+    const uint32_t n = back ? self : (uint32_t)(rowb[1 + ey] + col[1 + ex]);
+    const int di = back ? OPPd(i) : i;
+    const uint32_t base = K * n - (K - 2) * (n & 31u);
+    if constexpr (F32) {
+      LB_GUARD((unsigned long long)base + 64 * di + 1, lim, );
+      *reinterpret_cast<float2*>(dst.f + base + 64 * di) = make_float2(fs[i], ge[i]);
+    } else {
+      LB_GUARD((unsigned long long)base + 32 + 64 * (di - 1) + 1, lim, );
+      *reinterpret_cast<__half2*>(dst.f + base + 32 + 64 * (di - 1)) = __floats2half2_rn(fs[i], ge[i]);
+    }
+  }
+}
+
 // ---------------------------------------------------------------- the step
 
 template <int MODEL, class S>
@@ -1247,7 +1304,14 @@ __device__ __forceinline__ void step_strip(const Geom& G, const Phys<typename S:
   auto load = [&](int r, A* f, A* g) {
     const int rr = wrapi(r, ny);
     const bool fluid = !(tc[1] && !row_in_band(G, rr));
-    if (fluid) load_node<MODEL, S, false, RAW>(src, N, (size_t)rr * nx + x, f, g);
+    if (fluid) {
+      if constexpr (is_blocked<S>::value) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) S::lfg(src.f, src.g0, N, (size_t)rr * nx + x, i, f[i], g[i]);
+      } else {
+        load_node<MODEL, S, false, RAW>(src, N, (size_t)rr * nx + x, f, g);
+      }
+    }
     return fluid;
   };
   auto sums = [&](const A* f, const A* g, bool fluid) {
@@ -1306,7 +1370,10 @@ __device__ __forceinline__ void step_strip(const Geom& G, const Phys<typename S:
         collide_node<MODEL, A>(P, vr, vp, sol, bnd, fa, fs, ge);
       const int rowb[3] = {ym * nx, yy * nx, yp * nx};
       const int col[3] = {xm, x, xp};
-      push_node<MODEL, S, RAW>(dst, N, rowb, col, sol, bnd, fs, ge);
+      if constexpr (is_blocked<S>::value)
+        push_node_blk_rows<MODEL, S>(dst, (unsigned long long)(N + 31) / 32 * S::kBlock, rowb, col, sol, bnd, fs, ge);
+      else
+        push_node<MODEL, S, RAW>(dst, N, rowb, col, sol, bnd, fs, ge);
     }
     if (more) {
       Rw[0] = Rw[1];

@@ -402,41 +402,6 @@ __device__ __forceinline__ void push_node_blk16(__half* __restrict__ f, float* _
   }
 }
 
-// The same pairs when rows start inside blocks (nx % 32 != 0): a node's address takes
-// three operations, with 32 b = n - n % 32 (B floats or halves per block, the pairs 2 wide)
-// B (n / 32) + 2 (n % 32) = (B / 32) n - (B / 32 - 2) (n % 32).
-template <int MODEL, class S>
-__device__ __forceinline__ void push_node_blk_rows(const Buf<S>& dst, unsigned long long lim, const int rowb[3],
-                                                   const int col[3], const bool sol[3][3], bool bnd,
-                                                   const float fs[9], const float ge[9]) {
-  static_assert(MODEL == MODEL_BINARY, "the block storages hold the binary model");
-  constexpr bool F32 = std::is_same<S, SF32B>::value;
-  constexpr uint32_t K = S::kBlock / 32;
-  const uint32_t self = (uint32_t)(rowb[1] + col[1]);
-  if constexpr (!F32) {
-    const uint32_t r = self & 31u;
-    LB_GUARD(K * self - (K - 1) * r, lim, );
-    dst.f[K * self - (K - 1) * r] = __float2half_rn(fs[0]);
-    LB_GUARD((self >> 5) * SF16B::kG0Stride + r, lim / 2 - SF16B::kG0, );
-    dst.g0[(self >> 5) * SF16B::kG0Stride + r] = ge[0];
-  }
-#pragma unroll
-  for (int i = F32 ? 0 : 1; i < 9; ++i) {
-    const int ex = EXd(i), ey = EYd(i);
-    const bool back = bnd && sol[1 + ey][1 + ex];
-    const uint32_t n = back ? self : (uint32_t)(rowb[1 + ey] + col[1 + ex]);
-    const int di = back ? OPPd(i) : i;
-    const uint32_t base = K * n - (K - 2) * (n & 31u);
-    if constexpr (F32) {
-      LB_GUARD((unsigned long long)base + 64 * di + 1, lim, );
-      *reinterpret_cast<float2*>(dst.f + base + 64 * di) = make_float2(fs[i], ge[i]);
-    } else {
-      LB_GUARD((unsigned long long)base + 32 + 64 * (di - 1) + 1, lim, );
-      *reinterpret_cast<__half2*>(dst.f + base + 32 + 64 * (di - 1)) = __floats2half2_rn(fs[i], ge[i]);
-    }
-  }
-}
-
 // UROWS: block storage with rows that start inside a block (nx % 32 != 0): the
 // stage columns of a lane change from row to row (a separate instantiation, so
 // that aligned rows keep constant columns and no per-row work).
