@@ -354,7 +354,8 @@ static lb_status default_state(lb_ctx* c) {
 //   2048 x 64 FP32 planes         27.1   5.7 (64 x 2)       FP32 blocks  13.6   5.3 (64 x 2)
 //   4096 x 128 FP32 blocks        17.6  11.2 (128 x 6)      moments      15.0  11.3 (128 x 6)
 //   16384 x 256 FP32 blocks       85.4  79.6 (128 x 8)      moments      50.5  48.2 (128 x 12)
-//   16384 x 256 FP32 planes       97.0  90.5 (256 x 8)      FP64         888   838 (64 x 10)
+//   16384 x 256 FP32 planes       97.0  90.5 (256 x 8)      FP64         888   662 (64 x 10)
+//   (the liquid-gas FP64 figures with the collision as it is now; 128 x 16 before it)
 static void default_tile(lb_ctx* c) {
   const int nx = c->grid.nx, ny = c->grid.ny, st = c->prm.storage;
   const bool lg = c->prm.model == LB_MODEL_LIQUID_GAS;
@@ -388,11 +389,10 @@ static void default_tile(lb_ctx* c) {
     per_sm = 5;
     most = 12;
   } else if (st == LB_STORAGE_F64) {
-    // the FP64 pipe bounds these: narrow tiles spread it evenly (binary: its stages
-    // leave two CTAs per SM, at twice the width)
-    bx = cols = lg ? 64 : 128;
-    per_sm = lg ? 8 : 2;
-    most = lg ? 10 : 12;
+    // the FP64 pipe bounds these: short bands, which spread over the SMs evenly, up to
+    // several waves (the binary stages leave two CTAs per SM)
+    per_sm = lg ? 4 : 2;
+    most = 10;
   } else {
     // planar storages: wide tiles, whose longer copies suit the copy engine, unless they
     // leave SMs without a tile
@@ -410,6 +410,12 @@ static void default_tile(lb_ctx* c) {
   const double y = ceil(rows / (per_sm * device_sm_count()));
   c->tile_x = bx;
   c->tile_y = y < most ? (y < 1 ? 1 : (int)y) : most;
+  if (st == LB_STORAGE_F64 && auto_staged(c)) {
+    // us per step: 4096 x 128 liquid-gas 105.1, 102.5 and binary 197, 172 at the one-wave
+    // band and at four rows; 16384 x 256 662 at 64 x 10 and 668 at 128 x 8 (liquid-gas)
+    if (y > 5 && y <= 16 && c->tile_y > 4) c->tile_y = 4;
+    if (lg && y > 16 && nx > 64) c->tile_x = 64;
+  }
   if (c->tile_y > ny) c->tile_y = ny;
 }
 

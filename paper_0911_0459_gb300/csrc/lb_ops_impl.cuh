@@ -20,14 +20,14 @@ static inline Geom to_geom(const OpArgs& a) {
 }
 
 template <typename A>
-static Phys<A> to_phys(const OpArgs& a) {
+static Phys<A> to_phys(const OpArgs& a, bool lg) {
   Phys<A> p;
   p.kappa = A(a.kappa); p.a = A(a.a); p.b = A(a.b); p.T = A(a.T);
   p.Acoef = A(a.Acoef); p.M = A(a.M); p.nu_l = A(a.nu_l); p.nu_g = A(a.nu_g);
   p.nu = A(a.nu); p.lambda_scale = A(a.lambda_scale); p.h = A(a.h);
   p.lut = A(a.lut);
   p.lut_inv = a.lut > 0 ? A(1.0 / a.lut) : A(0);
-  p.omega = A(2.0 / (6.0 * a.nu + 1.0));
+  set_pair_constants(p, a.kappa, a.M, a.nu, a.lambda_scale, lg);
   return p;
 }
 
@@ -74,7 +74,7 @@ template <int MODEL, class S, int BX>
 static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
   StepArgs<MODEL, S> k;
   k.G = to_geom(a);
-  k.P = to_phys<typename S::A>(a);
+  k.P = to_phys<typename S::A>(a, MODEL == MODEL_LG);
   k.Q = mom_phys(a.kappa, a.Acoef, a.M, a.nu_l, a.nu_g, a.lambda_scale, a.h, a.lut);
   k.src = to_buf<S>(a.src, a);
   k.dst = to_buf<S>(a.dst, a);
@@ -99,7 +99,7 @@ static cudaError_t launch_staged(const OpArgs& a, cudaStream_t s) {
   }
   TmaArgs<MODEL, S> k;
   k.G = to_geom(a);
-  k.P = to_phys<typename S::A>(a);
+  k.P = to_phys<typename S::A>(a, MODEL == MODEL_LG);
   k.Q = mom_phys(a.kappa, a.Acoef, a.M, a.nu_l, a.nu_g, a.lambda_scale, a.h, a.lut);
   k.src = to_buf<S>(a.src, a);
   k.dst = to_buf<S>(a.dst, a);
@@ -154,7 +154,7 @@ cudaError_t ops_impl(OpKind op, const OpArgs& a, cudaStream_t s) {
       }
       return cudaErrorInvalidValue;
     case OP_INIT:
-      init_kernel<MODEL, S><<<grid_for(N, 256), 256, 0, s>>>(G, to_phys<A>(a), to_buf<S>(a.dst, a), a.in0, a.in1,
+      init_kernel<MODEL, S><<<grid_for(N, 256), 256, 0, s>>>(G, to_phys<A>(a, MODEL == MODEL_LG), to_buf<S>(a.dst, a), a.in0, a.in1,
                                                               a.in2, a.in3, a.in_cols ? size_t(0) : size_t(a.nx));
       return cudaGetLastError();
     case OP_FIELDS:

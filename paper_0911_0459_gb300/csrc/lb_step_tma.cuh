@@ -451,7 +451,9 @@ __device__ bool consume_tile(const Ring<MODEL, S, BX, NS>& R, const Geom& G, con
   // neighbours (taken once per row, when the row is summed).
   struct Row {
     A rc, rl, rr, pc, pl, pr;
+    RowSum wr, wp;  // FP64: the row's summaries (collide_pairs)
   };
+  constexpr bool PAIRS = std::is_same<A, double>::value;  // populations kept in pair form
   // extra column of the edge lanes: left neighbour of lane 0, right of lane 31
   const int sx = lane == 0 ? sc - 1 : sc + 1;
   // One value of a staged row for the halo sums: population i >= 1 of f (isg false)
@@ -499,12 +501,17 @@ __device__ bool consume_tile(const Ring<MODEL, S, BX, NS>& R, const Geom& G, con
     if (skip) {
       Rw.rc = Rw.rl = Rw.rr = A(0);
       Rw.pc = Rw.pl = Rw.pr = A(0);
+      if constexpr (PAIRS) Rw.wr = Rw.wp = RowSum{0.0, 0.0, 0.0, 0.0};
       return;
     }
     int co = sc, ce = sx;
     if constexpr (BR) row_cols(yr, co, ce);
     load_pop(s, co, f, g);
-    const A r = sum9(f);
+    A r;
+    if constexpr (PAIRS)
+      r = to_pairs(f);
+    else
+      r = sum9(f);
     const A p = BIN ? sum9(g) : A(0);
     int cl = warp * 32 + L::HALO - 1, cr = warp * 32 + L::HALO + 32;  // the halo columns
     if constexpr (BR) {
@@ -533,6 +540,10 @@ __device__ bool consume_tile(const Ring<MODEL, S, BX, NS>& R, const Geom& G, con
       Rw.pc = p;
       Rw.pl = lane == 0 ? pe : pl;
       Rw.pr = lane == 31 ? pe : pr;
+    }
+    if constexpr (PAIRS) {
+      Rw.wr = row_sum(Rw.rl, Rw.rc, Rw.rr);
+      if (BIN) Rw.wp = row_sum(Rw.pl, Rw.pc, Rw.pr);
     }
   };
 
@@ -654,19 +665,31 @@ __device__ bool consume_tile(const Ring<MODEL, S, BX, NS>& R, const Geom& G, con
 #pragma unroll
             for (int i = 0; i < 3; ++i) sol[j][i] = false;
         }
-        if constexpr (RAW)
+        if constexpr (RAW) {
           collide_node_f16<MODEL>(Q, vr, vp, sol, bnd, fa, fs, ge);
-        else
+        } else if constexpr (PAIRS) {
+          if (bnd) {
+            collide_pairs_node<MODEL>(P, vr, vp, sol, true, fa, fs, ge);
+          } else {
+            const RowSum wr[3] = {Rw[0].wr, Rw[1].wr, Rw[2].wr}, wp[3] = {Rw[0].wp, Rw[1].wp, Rw[2].wp};
+            collide_pairs<MODEL>(P, wr, wp, false, fa, fs, ge);
+          }
+        } else {
           collide_node<MODEL, A>(P, vr, vp, sol, bnd, fa, fs, ge);
+        }
         push(rowb, sol, bnd, fs, ge);
       }
     } else {
       const bool sol[3][3] = {{false, false, false}, {false, false, false}, {false, false, false}};
       if (act) {
-        if constexpr (RAW)
+        if constexpr (RAW) {
           collide_node_f16<MODEL>(Q, vr, vp, sol, false, fa, fs, ge);
-        else
+        } else if constexpr (PAIRS) {
+          const RowSum wr[3] = {Rw[0].wr, Rw[1].wr, Rw[2].wr}, wp[3] = {Rw[0].wp, Rw[1].wp, Rw[2].wp};
+          collide_pairs<MODEL>(P, wr, wp, false, fa, fs, ge);
+        } else {
           collide_node<MODEL, A>(P, vr, vp, sol, false, fa, fs, ge);
+        }
         push(rowb, sol, false, fs, ge);
       }
     }
@@ -708,6 +731,10 @@ __device__ __forceinline__ bool tile_all_solid(const Geom& G, int xb, int w, int
 // (each CTA with its 1 KB reservation), but no more than leaves 72 registers per
 // thread: the FP32 blocks at 128 columns and 4 stages fit four CTAs, which gives
 // 96 registers instead of the 72 of a five-CTA bound (1 % faster on 16384 x 256).
+// The FP64 storages, which the FP64 pipe bounds, get 128 registers, at which neither
+// model spills: the binary stages leave room for two CTAs of 128 columns anyway (at 72
+// registers it spilled 680 bytes a thread: 4096 x 128 189 -> 170 us), the liquid-gas
+// model needs no more than three (16384 x 256 676 -> 662 us against 80 registers).
 constexpr int tma_min_blocks(int bx, int ns) {
   return bx == 64 ? (ns > 4 ? 4 : 8) : (bx == 128 ? (ns > 4 ? 3 : 5) : (ns > 3 ? 2 : 3));
 }
@@ -719,6 +746,11 @@ constexpr int tma_min_blocks_of() {
     constexpr int by_regs = 65536 / ((BX + 32) * 72);
     constexpr int b = by_smem < by_regs ? by_smem : by_regs;
     return b < 1 ? 1 : (b > 8 ? 8 : b);
+  } else if constexpr (std::is_same<S, SF64>::value) {
+    constexpr int by_smem = int(233472 / (L::BYTES + 1024));
+    constexpr int by_regs = 65536 / ((BX + 32) * 128);
+    constexpr int b = by_smem < by_regs ? by_smem : by_regs;
+    return b < 1 ? 1 : b;
   } else {
     return tma_min_blocks(BX, NS);
   }
