@@ -37,7 +37,10 @@ inline void populate_host(const HostRange* r, int n) {
   constexpr size_t kPerThread = 2 << 20;  // a thread costs about as much to start as 0.5 MB of pages
   constexpr int kThreads = 4;  // more wait for one another in the kernel (134 MB: 3.9, 2.2, 1.5 ms with 1, 2, 4; 2.9 with 8)
   const size_t page = (size_t)sysconf(_SC_PAGESIZE);
-  if (page == 0) return;
+  size_t total = 0;
+  for (int i = 0; i < n; ++i)
+    if (r[i].p) total += r[i].bytes;
+  if (page == 0 || total < kLeast) return;
   // whether a range looks fresh: none of four of its pages in memory
   auto fresh = [=](const HostRange& x) {
     const uintptr_t a = ((uintptr_t)x.p + page - 1) / page, b = ((uintptr_t)x.p + x.bytes) / page;
@@ -49,7 +52,7 @@ inline void populate_host(const HostRange* r, int n) {
   };
   HostRange todo[kMost];
   int m = 0;
-  size_t total = 0;
+  total = 0;
   for (int i = 0; i < n && m < kMost; ++i)
     if (r[i].p && fresh(r[i])) {
       todo[m++] = r[i];

@@ -12,9 +12,8 @@
 // adds the FP32 partials in a fixed order (split-K, deterministic).
 // Epilogues fuse the bias and tanh (forward), the loss and its derivative, the
 // tanh derivative (backward) and the BF16 rounding of activations.  Ensemble
-// members run in the z dimension of every launch.  One training iteration (forward,
-// loss, backward, AdamW: seven launches) is captured once as a CUDA graph and
-// replayed.
+// members run in the z dimension of every launch.  Sixteen training iterations
+// (forward, loss, backward, AdamW) are captured once as a CUDA graph and replayed.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -24,6 +23,7 @@
 #include <string.h>
 
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "lb_host.h"
@@ -41,6 +41,7 @@ constexpr int kGemmSmem = kStages * 2 * kTileBytes;  // 48 KB: no opt-in, four C
 constexpr int kWgradStages = 6;     // the weight gradients' long K: 96 KB in flight, two CTAs per SM
 constexpr int kWgradThreads = 128;  // four warps of 32x32 (eight of 32x16: 38 instead of 33 us)
 constexpr int kWgradSmem = kWgradStages * 2 * kTileBytes;
+constexpr int kGraphSteps = 16;  // training steps per captured graph: the gap between graphs is 3 us (88 -> 85 us a step)
 constexpr int kBiasGroups = 8;  // partial sums of a bias gradient (32 row classes each)
 
 enum { EPI_BIAS_F32 = 0, EPI_BIAS_TANH = 1, EPI_LOSS = 2, EPI_DTANH = 3, EPI_PART = 4 };
@@ -79,6 +80,12 @@ __device__ __forceinline__ void mma_bf16(float c[4], const uint32_t a[4], const 
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
+
+// The kernels of a training step and of a prediction follow one another with programmatic
+// stream serialisation: the next one's CTAs may start while the last ones of this one
+// drain, and wait here before they touch memory.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <bool TRANS>
 __device__ __forceinline__ void ldmatrix4(uint32_t r[4], uint32_t addr) {
@@ -180,7 +187,7 @@ __device__ __forceinline__ void gemm_tile(const bf16* A, long lda, int M, const 
     cp_commit();
   };
 #pragma unroll
-  for (int c = 0; c < ST - 1; ++c) load(c);
+  for (int c = 0; c < ST - (SPLIT ? 2 : 1); ++c) load(c);
   const int l8 = lane & 7, li = lane >> 3;
   [[maybe_unused]] float run[2][NI][4];
   [[maybe_unused]] int next = kc;  // rows after which the running sum takes the accumulators
@@ -192,10 +199,15 @@ __device__ __forceinline__ void gemm_tile(const bf16* A, long lda, int M, const 
 #pragma unroll
         for (int k = 0; k < 4; ++k) run[i][j][k] = 0.0f;
   }
+  // chunks per barrier: two where the ring is deep (SPLIT)
+  constexpr int PER = SPLIT ? 2 : 1;
   for (int c = 0; c < nk; ++c) {
-    cp_wait<ST - 2>();
-    __syncthreads();
-    load(c + ST - 1);
+    if (PER == 1 || c % PER == 0) {
+      cp_wait<ST - 2 * PER>();
+      __syncthreads();
+#pragma unroll
+      for (int p = 0; p < PER; ++p) load(c + ST - PER + p);
+    }
     const uint32_t sa = rd, sbb = rd + kTileBytes;
     rd = rd == sb + (ST - 1) * 2 * kTileBytes ? sb : rd + 2 * kTileBytes;
     const int steps = min((ke - kb - c * TK + 15) / 16, TK / 16);
@@ -509,6 +521,7 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_kernel(RowsArgs a) {
   unsigned char* const dyp = smem + (dy - s0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, gq = lane >> 2, tq = lane & 3;
   const int nw = warp * 8 * NF;  // this warp's columns of the hidden layers
+  pdl_wait();
   // this CTA's member and its run of the member's tiles
   const int mem = blockIdx.x % a.members, slot = blockIdx.x / a.members, slots = gridDim.x / a.members;
   const long per = (a.n + R - 1) / R;
@@ -693,6 +706,22 @@ __global__ void __launch_bounds__(kRowThreads, 1) rows_kernel(RowsArgs a) {
     if (lane == 0) atomicAdd(a.loss + mem, lsum * a.scale);
     if (tid < R) bulk_wait_all();
   }
+  pdl_trigger();
+}
+
+template <class... P, class... A>
+static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 template <int NT, int RT, bool TRAIN>
@@ -700,8 +729,8 @@ static cudaError_t launch_rows_at(const RowsArgs& a, size_t smem, int sms, cudaS
   cudaError_t e = cudaFuncSetAttribute(rows_kernel<NT, RT, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e) return e;
   const long tiles = (a.n + 16 * RT - 1) / (16 * RT), slots = sms / a.members > 1 ? sms / a.members : 1;
-  rows_kernel<NT, RT, TRAIN><<<(unsigned)(a.members * (tiles < slots ? tiles : slots)), kRowThreads, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(rows_kernel<NT, RT, TRAIN>, dim3((unsigned)(a.members * (tiles < slots ? tiles : slots))), kRowThreads,
+                    smem, s, a);
 }
 template <int RT, bool TRAIN>
 static cudaError_t launch_rows_of(const RowsArgs& a, int nh, size_t smem, int sms, cudaStream_t s) {
@@ -784,6 +813,7 @@ __device__ __forceinline__ void bias_group(const float* X, int rows, int cols, i
 
 __global__ void __launch_bounds__(kWgradThreads) wgrad_kernel(WgradArgs a) {
   extern __shared__ __align__(128) unsigned char smem[];
+  pdl_wait();
   if (a.sc && blockIdx.x == 0 && threadIdx.x == 0) a.sc->t += 1;
   // the products first (they take longest): member, then split, then tile
   int t = blockIdx.x;
@@ -883,6 +913,7 @@ __global__ void __launch_bounds__(256) adamw_kernel(float* p, bf16* pb, const fl
                                                     float* m1, float* m2, long P, const Sched* sc, Offsets o,
                                                     float* loss) {
   const int mem = blockIdx.y;
+  pdl_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0) loss[mem] = 0.0f;  // for the next step
   const int t = sc->t + 1;
   const float pi = 3.14159265358979f;
@@ -972,6 +1003,7 @@ __global__ void init_params_kernel(float* p, bf16* pb, long P, unsigned long lon
 // (count, the member stride and the arrays are multiples of 16 bytes).
 __global__ void __launch_bounds__(256) ensemble_kernel(const float* Y, int K, long stride, long count, float* mean,
                                                        float* sd) {
+  pdl_wait();
   for (long e = 4 * (blockIdx.x * (long)blockDim.x + threadIdx.x); e < count; e += 4L * gridDim.x * blockDim.x) {
     float s[4] = {0.0f, 0.0f, 0.0f, 0.0f}, q[4] = {0.0f, 0.0f, 0.0f, 0.0f}, mu[4], dv[4];
     for (int k = 0; k < K; ++k) {
@@ -1257,8 +1289,7 @@ static cudaError_t backward(lb_mlp* m, Sched* sc, cudaStream_t s) {
   if (e) return e;
   const unsigned blocks = (unsigned)m->K * ((unsigned)(a.tiles[0] + a.tiles[1] + a.tiles[2]) * a.parts +
                                             (unsigned)(a.bblocks[0] + a.bblocks[1] + a.bblocks[2]) * kBiasGroups);
-  wgrad_kernel<<<blocks, kWgradThreads, kWgradSmem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(wgrad_kernel, dim3(blocks), kWgradThreads, kWgradSmem, s, a);
 }
 
 static Offsets offsets(const lb_mlp* m) {
@@ -1271,9 +1302,7 @@ static cudaError_t train_step(lb_mlp* m, cudaStream_t s) {
   int ks, kc;
   wgrad_splits(m, m->n, &ks, &kc);
   ks = wgrad_parts(m, ks);
-  adamw_kernel<<<dim3((unsigned)((m->P / 4 + 255) / 256), m->K), 256, 0, s>>>(m->p, m->pb, m->part, m->bpart, ks, m->m1,
-                                                                           m->m2, m->P, m->sched, offsets(m), m->loss);
-  return cudaGetLastError();
+  return launch_pdl(adamw_kernel, dim3((unsigned)((m->P / 4 + 255) / 256), m->K), 256, 0, s, m->p, m->pb, (const float*)m->part, (const float*)m->bpart, ks, m->m1, m->m2, m->P, (const Sched*)m->sched, offsets(m), m->loss);
 }
 
 extern "C" {
@@ -1435,9 +1464,10 @@ lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, f
   if (!m || steps < 1 || m->n < 1 || !(lr > 0)) return LB_ERR_ARG;
   Sched sc = {-1, steps, lr, lr_min, wd};  // every step's gradient launch counts it
   MCK(cudaMemcpyAsync(m->sched, &sc, sizeof sc, cudaMemcpyHostToDevice, m->stream));
-  if (!m->gexec) {
+  if (!m->gexec && steps >= kGraphSteps) {
     MCK(cudaStreamBeginCapture(m->cap, cudaStreamCaptureModeThreadLocal));
-    cudaError_t e = train_step(m, m->cap);
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < kGraphSteps && e == cudaSuccess; ++k) e = train_step(m, m->cap);
     cudaGraph_t g = NULL;
     cudaError_t e2 = cudaStreamEndCapture(m->cap, &g);
     if (e == cudaSuccess) e = e2;
@@ -1446,7 +1476,8 @@ lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, f
     if (e != cudaSuccess) return merr(m, "graph capture failed: %s", cudaGetErrorString(e)), LB_ERR_CUDA;
   }
   MCK(cudaMemsetAsync(m->loss, 0, m->K * sizeof(float), m->stream));
-  for (int i = 0; i < steps; ++i) MCK(cudaGraphLaunch(m->gexec, m->stream));
+  for (int i = 0; i < steps / kGraphSteps; ++i) MCK(cudaGraphLaunch(m->gexec, m->stream));
+  for (int i = 0; i < steps % kGraphSteps; ++i) MCK(train_step(m, m->stream));
   if (losses) {
     // loss of the final parameters (the last update cleared the sums)
     const int rt = rows_plan(m, m->n, true);
@@ -1469,9 +1500,8 @@ lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* s
     MCK(cudaGetLastError());
     MCK(forward(m, n, m->xbp, false, m->stream));
   }
-  ensemble_kernel<<<blocks_for(m, (long)n * m->nout / 4), 256, 0, m->stream>>>(
-      m->y, m->K, (long)m->maxb * m->nout, (long)n * m->nout, m->mean, m->sd);
-  MCK(cudaGetLastError());
+  MCK(launch_pdl(ensemble_kernel, dim3(blocks_for(m, (long)n * m->nout / 4)), 256, 0, m->stream, (const float*)m->y,
+                 m->K, (long)m->maxb * m->nout, (long)n * m->nout, m->mean, m->sd));
   const size_t out = (size_t)n * m->nout * 4;
   const lbk::HostRange host[3] = {{mean, out}, {sd, out}, {members, out * m->K}};
   lbk::populate_host(host, 3);  // beside the kernels
