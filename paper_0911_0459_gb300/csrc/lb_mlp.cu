@@ -1054,7 +1054,9 @@ struct lb_mlp {
   int n;  // rows of the loaded data
   int sms;          // SMs of the device and shared memory a block may opt in to
   size_t max_smem;
-  float *xin, *mean, *sd;  // host rows on their way in, ensemble statistics on their way out
+  // host rows on their way in and ensemble statistics on their way out: in buffers that only
+  // a backward pass uses (one member's mean is its output)
+  float *xin, *mean, *sd;
   cudaGraphExec_t gexec;
   int graph_n;
   char err[512];
@@ -1349,9 +1351,6 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
   m->loss = (float*)malloc_dev(m, 64 * sizeof(float));
   m->xb = (bf16*)malloc_dev(m, B * 16 * 2);
   m->xbp = (bf16*)malloc_dev(m, B * 16 * 2);
-  m->xin = (float*)malloc_dev(m, B * nin * 4);
-  m->mean = (float*)malloc_dev(m, B * nout * 4);
-  m->sd = (float*)malloc_dev(m, B * nout * 4);
   m->h1 = (bf16*)malloc_dev(m, members * B * nh * 2);
   m->h2 = (bf16*)malloc_dev(m, members * B * nh * 2);
   m->dz2b = (bf16*)malloc_dev(m, members * B * nh * 2);
@@ -1371,10 +1370,13 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
     const long cap = (256L << 20) / (4L * members * mn);
     if (ks > cap) ks = cap;
     m->ks_max = ks > 1 ? (int)ks : 1;
-    m->part = (float*)malloc_dev(m, 4L * members * m->ks_max * m->P);
+    m->part = (float*)malloc_dev(m, 4L * members * wgrad_parts(m, m->ks_max) * m->P);
     m->bpart = (float*)malloc_dev(m, 4L * members * kBiasGroups * (2 * nh + nout));
   }
-  bool ok = m->part && m->bpart && m->p && m->g && m->m1 && m->m2 && m->pb && m->sched && m->loss && m->xb && m->xbp && m->xin && m->mean && m->sd && m->h1 && m->h2 && m->dz2b &&
+  m->xin = m->dz2f;
+  m->mean = members > 1 ? m->dyf : m->y;
+  m->sd = members > 1 && m->dyf ? m->dyf + B * nout : m->dyf;
+  bool ok = m->part && m->bpart && m->p && m->g && m->m1 && m->m2 && m->pb && m->sched && m->loss && m->xb && m->xbp && m->h1 && m->h2 && m->dz2b &&
             m->dz1b && m->dz2f && m->dz1f && m->y && m->dyf && m->dyb && m->t;
   if (!ok) {
     lb_mlp_destroy(m);
