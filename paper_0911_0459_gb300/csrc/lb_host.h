@@ -6,7 +6,9 @@
 // populate_host asks the system for the pages beforehand, beside the kernels that still
 // run and by several threads where there are many (5.4 ms and 0.26 ms).  It changes no
 // byte: pages that exist stay as they are, ranges whose pages exist already are left
-// alone (asking for 134 MB of them takes 1.4 ms), and where the system does not know the
+// alone (asking for 134 MB of them takes 1.4 ms), a range that has some of them is asked for
+// whole (predictions of 65536 rows into arrays that a heap hands out again, 33.5 MB: 1443 ->
+// 1051 us against looking at four pages only), and where the system does not know the
 // request or the address the copy finds what it found before.
 #pragma once
 
@@ -30,8 +32,8 @@ struct HostRange {
 };
 
 // Pages wholly inside the ranges (the first and last partial page hold other data too and
-// usually exist; the copy faults them in otherwise).
-inline void populate_host(const HostRange* r, int n) {
+// usually exist; the copy faults them in otherwise).  True if there were any to make.
+inline bool populate_host(const HostRange* r, int n) {
   constexpr int kMost = 4;                // ranges looked at
   constexpr size_t kLeast = 1 << 20;      // smaller results: sixteen faults at most, or memory in use already
   constexpr size_t kPerThread = 2 << 20;  // a thread costs about as much to start as 0.5 MB of pages
@@ -40,15 +42,19 @@ inline void populate_host(const HostRange* r, int n) {
   size_t total = 0;
   for (int i = 0; i < n; ++i)
     if (r[i].p) total += r[i].bytes;
-  if (page == 0 || total < kLeast) return;
-  // whether a range looks fresh: none of four of its pages in memory
+  if (page == 0 || total < kLeast) return false;
+  // whether a page of the range is not in memory (a heap that shrank and grew again has its
+  // first page, and a result that was used in part others)
   auto fresh = [=](const HostRange& x) {
     const uintptr_t a = ((uintptr_t)x.p + page - 1) / page, b = ((uintptr_t)x.p + x.bytes) / page;
-    for (uintptr_t k = 0; b > a && k < 4; ++k) {
-      unsigned char in = 0;
-      if (mincore((void*)((a + (b - a - 1) * k / 3) * page), page, &in) != 0 || (in & 1)) return false;
+    unsigned char in[1024];
+    for (uintptr_t k = a; k < b; k += sizeof in) {
+      const size_t cnt = b - k < sizeof in ? b - k : sizeof in;
+      if (mincore((void*)(k * page), cnt * page, in) != 0) return false;
+      for (size_t q = 0; q < cnt; ++q)
+        if (!(in[q] & 1)) return true;
     }
-    return b > a;
+    return false;
   };
   HostRange todo[kMost];
   int m = 0;
@@ -58,7 +64,7 @@ inline void populate_host(const HostRange* r, int n) {
       todo[m++] = r[i];
       total += r[i].bytes;
     }
-  if (total < kLeast) return;
+  if (total < kLeast) return false;
   // part k of parts: the same share of every range
   auto part = [&todo, m, page](int k, int parts) {
     for (int i = 0; i < m; ++i) {
@@ -77,10 +83,11 @@ inline void populate_host(const HostRange* r, int n) {
   }
   for (int k = started; k < parts; ++k) part(k, parts);
   for (int i = 0; i < started; ++i) t[i].join();
+  return true;
 }
-inline void populate_host(void* p, size_t bytes) {
+inline bool populate_host(void* p, size_t bytes) {
   const HostRange r = {p, bytes};
-  populate_host(&r, 1);
+  return populate_host(&r, 1);
 }
 
 }  // namespace lbk

@@ -18,7 +18,7 @@ torch = pytest.importorskip("torch")
 if not torch.cuda.is_available():
     pytest.skip("no CUDA device", allow_module_level=True)
 
-from paper_0911_0459_gb300.mlp import MLP  # noqa: E402
+from paper_0911_0459_gb300.mlp import MLP, _lib, _ptr  # noqa: E402
 from test_gpu_mlp import bf16_round  # noqa: E402
 
 
@@ -46,4 +46,25 @@ def test_gradients_and_predictions_at_the_edges_of_the_tiles(nin, nh, nout, memb
             assert err < 2e-2, (k, name, err)
         yr, _ = ref.forward(p, x.astype(np.float64), nin, nh, nout)
         assert np.linalg.norm(out[k] - yr) < 2e-2 * np.linalg.norm(yr)
+    net.close()
+
+
+@pytest.mark.parametrize("nin,nh,nout,members,n", [
+    (4, 256, 64, 5, 8192), (4, 256, 64, 5, 20011), (3, 64, 200, 1, 14593), (16, 192, 24, 16, 45000), (2, 128, 8, 7, 70000)])
+def test_large_predictions_equal_those_of_their_rows(nin, nh, nout, members, n):
+    """Results above 4 MB reach host arrays that exist in parts; a row's outputs do not depend
+    on the rows beside it, so they are the bytes that short predictions give (no tolerance)."""
+    rng = np.random.default_rng(n)
+    net = MLP(nin, nh, nout, members=members, max_batch=n, seed=2)
+    x = rng.uniform(-1, 1, (n, nin)).astype(np.float32)
+    out = [np.full((n, nout), np.nan, np.float32), np.full((n, nout), np.nan, np.float32),
+           np.full((members, n, nout), np.nan, np.float32)]
+    assert _lib().lb_mlp_predict(net.h, n, _ptr(x), *(_ptr(a) for a in out)) == 0
+    fresh = net.predict(x, members=True)
+    for a, b in zip(out, fresh):
+        assert np.array_equal(a, b)
+    for r in (0, n // 3, n // 2 - 7, n - 301):
+        mean, sd, each = net.predict(x[r:r + 301], members=True)
+        assert np.array_equal(mean, out[0][r:r + 301]) and np.array_equal(sd, out[1][r:r + 301])
+        assert np.array_equal(each, out[2][:, r:r + 301])
     net.close()
