@@ -373,14 +373,17 @@ static void default_tile(lb_ctx* c) {
     // (4097 x 128 FP32: 15.1, 16.0 us at 4, 8 rows; 16391 x 256: 103.8, 101.3 us)
     const double strips = (double)((nx + 29) / 30) * ((double)c->fluid / nx), wave = 15.0 * device_sm_count();
     const bool f64 = st == LB_STORAGE_F64, small = staged_ok(st, nx, ny) || strips <= 2 * wave;
-    if (!f64 || small) {
+    const bool wide = st != LB_STORAGE_F32_BLOCKED && st != LB_STORAGE_F16_BLOCKED && 9ull * nx * ny >= 1ull << 32;
+    if (!wide && (!f64 || small)) {
       const double y = ceil(strips / wave);
       c->tile_x = 64;
       c->tile_y = f64 ? (y < 2 ? 1 : 2) : (y <= 4 ? (y < 1 ? 1 : (int)y) : (strips > 16 * wave ? 8 : 4));
       if (c->tile_y > ny) c->tile_y = ny;
       return;
     }
-    per_sm = 4;  // FP64 at a width the staged kernel does not take: the shared window
+    // FP64 at a width the staged kernel does not take, planes beyond 32-bit offsets: the
+    // shared window
+    per_sm = 4;
     most = 24;
   } else if (st == LB_STORAGE_F32_BLOCKED) {
     per_sm = 4;

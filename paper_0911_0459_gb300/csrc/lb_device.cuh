@@ -197,6 +197,15 @@ struct SF32 {
     LB_GUARD(i * N + n, 9 * N, A(0));
     return __ldcg(g + i * N + n);
   }
+  // loads and stores at 32-bit element offsets
+  __device__ static A lfo(const T* __restrict__ f, uint32_t N, uint32_t n, int i, const Rest&) {
+    LB_GUARD((unsigned long long)i * N + n, 9ull * N, A(0));
+    return __ldg(f + (i * N + n));
+  }
+  __device__ static A lgo(const T* __restrict__ g, const float* __restrict__, uint32_t N, uint32_t n, int i) {
+    LB_GUARD((unsigned long long)i * N + n, 9ull * N, A(0));
+    return __ldg(g + (i * N + n));
+  }
   __device__ static void sfo(T* __restrict__ f, uint32_t N, uint32_t n, int i, A v, const Rest&) {
     LB_GUARD((unsigned long long)i * N + n, 9ull * N, );
     f[i * N + n] = v;
@@ -250,6 +259,13 @@ struct SF16 {
     else
       g[(i - 1) * N + n] = __float2half_rn(v);
   }
+  __device__ static A lfo(const T* __restrict__ f, uint32_t N, uint32_t n, int i, const Rest& r) {
+    return lfro(f, N, n, i) + rest_w(r, i);
+  }
+  __device__ static A lgo(const T* __restrict__ g, const float* __restrict__ g0, uint32_t N, uint32_t n, int i) {
+    LB_GUARD(i == 0 ? (unsigned long long)n : (unsigned long long)(i - 1) * N + n, i == 0 ? N : 8ull * N, A(0));
+    return i == 0 ? __ldg(g0 + n) : __half2float(__ldg(g + ((i - 1) * N + n)));
+  }
   __device__ static void sfo(T* __restrict__ f, uint32_t N, uint32_t n, int i, A v, const Rest& r) {
     LB_GUARD((unsigned long long)i * N + n, 9ull * N, );
     f[i * N + n] = __float2half_rn(v - rest_w(r, i));
@@ -267,6 +283,10 @@ struct SF16 {
   __device__ static A lfr(const T* __restrict__ f, size_t N, size_t n, int i) {
     LB_GUARD(i * N + n, 9 * N, A(0));
     return __half2float(__ldg(f + i * N + n));
+  }
+  __device__ static A lfro(const T* __restrict__ f, uint32_t N, uint32_t n, int i) {
+    LB_GUARD((unsigned long long)i * N + n, 9ull * N, A(0));
+    return __half2float(__ldg(f + (i * N + n)));
   }
   __device__ static A lfcr(const T* f, size_t N, size_t n, int i) {
     LB_GUARD(i * N + n, 9 * N, A(0));
@@ -926,7 +946,7 @@ __device__ __forceinline__ double to_pairs(double f[9]) {
 // fp: populations in pair form (to_pairs); at rest (boundary nodes, Sec. 2.2) the momentum
 // is zero, which the rest rule leaves the sums out of.  Every product that feeds a sum is an
 // explicit fused multiply-add or __dmul_rn, so that all kernels round alike.
-// The liquid-gas step takes about 92 FP64 operations a node instead of 120 with 3x3
+// The liquid-gas step takes 91 FP64 operations a node instead of 120 with 3x3
 // stencils and separate odd parts: 838 -> 662 us on 16384 x 256, 7.2 -> 6.0 us on 256 x 32;
 // binary 16384 x 256 1381 -> 1098 us.
 // (In FP32 on full population values this form moved phi beyond the method's bar; FP64
@@ -1366,7 +1386,9 @@ __device__ __forceinline__ void step_band(const Geom& G, const Phys<typename S::
 // the two idle lanes cost less than the barriers in FP32.  Us per step, shared window ->
 // strips, best tile of each: 704 x 40 FP32 planes 3.68 -> 2.76, 2048 x 64 6.43 -> 5.58,
 // 1000 x 200 8.14 -> 7.79, 16391 x 256 104.4 -> 101.3; 256 x 32 liquid-gas FP64 8.5 ->
-// 7.0 (its FP64 sums without the halo columns).
+// 7.0 (its FP64 sums without the halo columns).  FP32 and FP16 planes are addressed by 32-bit
+// element offsets (planes of 9 N >= 2^32 values take the shared window): 700 x 40 2.85 ->
+// 2.81, 2048 x 64 5.77 -> 5.66; the FP64 strips spilled with them.
 constexpr int kStripCols = 30;
 
 template <int MODEL, class S>
@@ -1395,8 +1417,18 @@ __device__ __forceinline__ void step_strip(const Geom& G, const Phys<typename S:
       if constexpr (is_blocked<S>::value) {
 #pragma unroll
         for (int i = 0; i < 9; ++i) S::lfg(src.f, src.g0, N, (size_t)rr * nx + x, i, f[i], g[i]);
+      } else if constexpr (std::is_same<A, double>::value) {
+        load_node<MODEL, S>(src, N, (size_t)rr * nx + x, f, g);
       } else {
-        load_node<MODEL, S, false, RAW>(src, N, (size_t)rr * nx + x, f, g);
+        const uint32_t n = (uint32_t)(rr * nx + x);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          if constexpr (RAW)
+            f[i] = S::lfro(src.f, (uint32_t)N, n, i);
+          else
+            f[i] = S::lfo(src.f, (uint32_t)N, n, i, src.r);
+          if (BIN) g[i] = S::lgo(src.g, src.g0, (uint32_t)N, n, i);
+        }
       }
     }
     return fluid;
@@ -1459,8 +1491,10 @@ __device__ __forceinline__ void step_strip(const Geom& G, const Phys<typename S:
       const int col[3] = {xm, x, xp};
       if constexpr (is_blocked<S>::value)
         push_node_blk_rows<MODEL, S>(dst, (unsigned long long)(N + 31) / 32 * S::kBlock, rowb, col, sol, bnd, fs, ge);
+      else if constexpr (std::is_same<A, double>::value)
+        push_node<MODEL, S>(dst, N, rowb, col, sol, bnd, fs, ge);
       else
-        push_node<MODEL, S, RAW>(dst, N, rowb, col, sol, bnd, fs, ge);
+        push_node_u32<MODEL, S, RAW>(dst, (uint32_t)N, rowb, col, sol, bnd, fs, ge);
     }
     if (more) {
       Rw[0] = Rw[1];

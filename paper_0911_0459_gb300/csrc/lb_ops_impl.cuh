@@ -79,8 +79,9 @@ static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
   k.src = to_buf<S>(a.src, a);
   k.dst = to_buf<S>(a.dst, a);
   k.yc = a.yc;
-  if constexpr (std::is_same<typename S::A, double>::value) {
-    if (a.yc > kStripRowsF64)
+  if constexpr (!is_blocked<S>::value) {
+    constexpr bool F64 = std::is_same<typename S::A, double>::value;
+    if (F64 ? a.yc > kStripRowsF64 : 9ull * a.nx * a.ny >= 1ull << 32)  // (FP32 strips: 32-bit offsets)
       return launch_pdl(step_kernel<MODEL, S, BX>, tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc), BX, 0, s, k);
   }
   return launch_pdl(strip_kernel<MODEL, S, BX / 32>,
