@@ -139,7 +139,7 @@ def step_kernel_label(variant, tx, ty, storage="FP32"):
                 f"(variant {variant}, tile {tx}x{ty})")
     if variant == 4:
         return f"moment_step_kernel<{storage}> (tile {tx}x{ty})"
-    return f"step_kernel<binary, {storage}, BX={tx}> (variant {variant}, tile {tx}x{ty})"
+    return f"strip_kernel<binary, {storage}, NW={tx // 32}> (variant {variant}, tile {tx}x{ty})"
 
 
 def ncu_traffic(kind, variant, tile):
@@ -160,10 +160,10 @@ def ncu_traffic(kind, variant, tile):
 
 
 # FP64 work per fluid-node update of the liquid-gas step kernel (ncu instruction counts of
-# one launch on 16384 x 256: 129.2 M DFMA, 82.6 M DMUL, 184.4 M DADD over 3 305 472 fluid
-# nodes): 120 FP64 instructions, 159 flops (an FMA counts two)
-LG_FP64_INST_PER_LU = 120.0
-LG_FP64_FLOPS_PER_LU = 159.0
+# one launch on 16384 x 256 at 64 x 10: 133.0 M DFMA, 56.1 M DMUL, 110.8 M DADD over 3 305 472
+# fluid nodes): 90.7 FP64 instructions, 131 flops (an FMA counts two)
+LG_FP64_INST_PER_LU = 90.7
+LG_FP64_FLOPS_PER_LU = 131.0
 
 
 def lg_fp64_roofline(torch, Lattice):
@@ -190,8 +190,8 @@ def lg_fp64_roofline(torch, Lattice):
            "frac_of_fp64_peak": achieved / rate,
            "frac_of_fp64_pipe": pipe / (rate / 2.0),
            "GBps": fluid * 144 / (ms * 1e-3) / 1e9,
-           "what": "liquid-gas FP64, 144 B/LU; FP64 flops per LU from ncu instruction counts (159: 39 DFMA, "
-                   "25 DMUL, 56 DADD); frac_of_fp64_pipe counts every FP64 instruction as one FMA slot"}
+           "what": "liquid-gas FP64, 144 B/LU; FP64 flops per LU from ncu instruction counts (131: 40 DFMA, "
+                   "17 DMUL, 34 DADD); frac_of_fp64_pipe counts every FP64 instruction as one FMA slot"}
     lat.close()
     return out
 
@@ -382,9 +382,9 @@ def batched_vs_sequential(torch, Lattice, steps, n=256, storage=None):
             "capillaries_per_s_at_20k_steps_extrapolated": cs_batch / 20000.0,
             "sequential_capillaries_per_s_at_20k_steps_extrapolated": cs_seq / 20000.0,
             "baselines": "single_lattice_path: each capillary its own lattice in the same storage on the "
-                         "library's default kernel and tile (the staged kernel where it applies, bands of 16 "
-                         "rows; 64-step CUDA graphs), run in turn; one_launch_per_run: each capillary alone "
-                         "in the batch's persistent kernel and tile (a batch of one), launched in turn",
+                         "library's default kernel and tile (chosen by lattice size; 64-step CUDA graphs), run "
+                         "in turn; one_launch_per_run: each capillary alone in the batch's persistent kernel "
+                         "and tile (a batch of one), launched in turn",
             "GLUPS_batched": fluid * steps / t_batch / 1e9, "fluid_nodes": fluid, "steps": steps,
             "tile": [tx, ty], "l_finite": bool(np.isfinite(out).all()),
             "what": f"{steps} steps with 4 l(t) samples, wall clock"}
