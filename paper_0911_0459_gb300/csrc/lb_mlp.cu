@@ -411,8 +411,8 @@ __global__ void __launch_bounds__(kGemmThreads) layer1_kernel(const bf16* x, con
 // n_hidden / 8 columns, so that a weight fragment read from shared memory (whose
 // bandwidth is the bound) serves three products.  Rows of shared memory are padded by
 // 16 bytes: the eight rows of one ldmatrix phase then lie in different banks.
-// 4096 rows x 5 members, n_hidden 256, n_out 64: 46 us for the forward pass, the loss
-// and the backward products, against 85 us as five launches of the GEMM kernel above
+// 4096 rows x 5 members, n_hidden 256, n_out 64: 42 us for the forward pass, the loss
+// and the backward products, against 88 us as five launches of the GEMM kernel above
 // (which takes the wider networks).  The tensor pipe is active a quarter of the time;
 // the rest is the FP32 gradients' stores, the tanh and the barriers between layers.
 struct RowsArgs {
