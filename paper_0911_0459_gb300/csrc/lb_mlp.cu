@@ -850,48 +850,57 @@ static cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, unsigned block, s
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
+// What a launch of the row kernels needs to know of the device.  The dynamic shared memory
+// limit belongs to a kernel, which every network of its n_hidden launches, from any thread:
+// all set it to the device's own limit (max_smem) and give the size they use to the launch.
+struct RowsDevice {
+  int sms;
+  size_t max_smem;
+};
+
 template <int NT>
-static cudaError_t launch_predict_at(const RowsArgs& a, size_t smem, int sms, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(predict_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+static cudaError_t launch_predict_at(const RowsArgs& a, size_t smem, const RowsDevice& d, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(predict_kernel<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.max_smem);
   if (e) return e;
-  const int slots = sms / a.members > 1 ? sms / a.members : 1;
+  const int slots = d.sms / a.members > 1 ? d.sms / a.members : 1;
   return launch_pdl(predict_kernel<NT>, dim3((unsigned)(a.members * slots)), kPredictThreads, smem, s, a);
 }
-static cudaError_t launch_predict(const RowsArgs& a, int nh, int sms, cudaStream_t s) {
+static cudaError_t launch_predict(const RowsArgs& a, int nh, const RowsDevice& d, cudaStream_t s) {
   const size_t smem = rows_smem(nh, a.nout, 3, false);
   switch (nh / 64) {
-    case 1: return launch_predict_at<1>(a, smem, sms, s);
-    case 2: return launch_predict_at<2>(a, smem, sms, s);
-    case 3: return launch_predict_at<3>(a, smem, sms, s);
-    case 4: return launch_predict_at<4>(a, smem, sms, s);
+    case 1: return launch_predict_at<1>(a, smem, d, s);
+    case 2: return launch_predict_at<2>(a, smem, d, s);
+    case 3: return launch_predict_at<3>(a, smem, d, s);
+    case 4: return launch_predict_at<4>(a, smem, d, s);
   }
   return cudaErrorInvalidValue;
 }
 
 template <int NT, int RT, bool TRAIN>
-static cudaError_t launch_rows_at(const RowsArgs& a, size_t smem, int sms, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(rows_kernel<NT, RT, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+static cudaError_t launch_rows_at(const RowsArgs& a, size_t smem, const RowsDevice& d, cudaStream_t s) {
+  cudaError_t e =
+      cudaFuncSetAttribute(rows_kernel<NT, RT, TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.max_smem);
   if (e) return e;
-  const long tiles = (a.n + 16 * RT - 1) / (16 * RT), slots = sms / a.members > 1 ? sms / a.members : 1;
+  const long tiles = (a.n + 16 * RT - 1) / (16 * RT), slots = d.sms / a.members > 1 ? d.sms / a.members : 1;
   return launch_pdl(rows_kernel<NT, RT, TRAIN>, dim3((unsigned)(a.members * (tiles < slots ? tiles : slots))), kRowThreads,
                     smem, s, a);
 }
 template <int RT, bool TRAIN>
-static cudaError_t launch_rows_of(const RowsArgs& a, int nh, size_t smem, int sms, cudaStream_t s) {
+static cudaError_t launch_rows_of(const RowsArgs& a, int nh, size_t smem, const RowsDevice& d, cudaStream_t s) {
   switch (nh / 64) {
-    case 1: return launch_rows_at<1, RT, TRAIN>(a, smem, sms, s);
-    case 2: return launch_rows_at<2, RT, TRAIN>(a, smem, sms, s);
-    case 3: return launch_rows_at<3, RT, TRAIN>(a, smem, sms, s);
-    case 4: return launch_rows_at<4, RT, TRAIN>(a, smem, sms, s);
+    case 1: return launch_rows_at<1, RT, TRAIN>(a, smem, d, s);
+    case 2: return launch_rows_at<2, RT, TRAIN>(a, smem, d, s);
+    case 3: return launch_rows_at<3, RT, TRAIN>(a, smem, d, s);
+    case 4: return launch_rows_at<4, RT, TRAIN>(a, smem, d, s);
   }
   return cudaErrorInvalidValue;
 }
 template <bool TRAIN>
-static cudaError_t launch_rows(const RowsArgs& a, int nh, int rt, int sms, cudaStream_t s) {
+static cudaError_t launch_rows(const RowsArgs& a, int nh, int rt, const RowsDevice& d, cudaStream_t s) {
   const size_t smem = rows_smem(nh, a.nout, rt, TRAIN);
   if constexpr (TRAIN)  // (predictions on tiles of 48 rows: launch_predict)
-    if (rt == 3) return launch_rows_of<3, true>(a, nh, smem, sms, s);
-  return launch_rows_of<1, TRAIN>(a, nh, smem, sms, s);
+    if (rt == 3) return launch_rows_of<3, true>(a, nh, smem, d, s);
+  return launch_rows_of<1, TRAIN>(a, nh, smem, d, s);
 }
 
 // Gradients of all weights and biases in one launch.  The batch rows are cut into ks
@@ -1198,8 +1207,7 @@ struct lb_mlp {
   float *part, *bpart;  // split-K partials of the weight gradients, row-class partials of the bias gradients
   int ks_max;           // largest K split the partial buffer holds
   int n;  // rows of the loaded data
-  int sms;          // SMs of the device and shared memory a block may opt in to
-  size_t max_smem;
+  RowsDevice dev;  // SMs of the device and shared memory a block may opt in to
   // host rows on their way in and ensemble statistics on their way out: in buffers that only
   // a backward pass uses (one member's mean is its output)
   float *xin, *mean, *sd;
@@ -1244,7 +1252,7 @@ static void* malloc_dev(lb_mlp* m, size_t bytes) {
 
 // Blocks of 256 threads for a grid-stride kernel over count items.
 static unsigned blocks_for(const lb_mlp* m, long count) {
-  const long b = (count + 255) / 256, most = 16L * m->sms;
+  const long b = (count + 255) / 256, most = 16L * m->dev.sms;
   return (unsigned)(b < 1 ? 1 : (b < most ? b : most));
 }
 
@@ -1260,8 +1268,8 @@ static cudaError_t gemm(const GemmArgs& g, int members, cudaStream_t s) {
 // spread over the SMs (512 rows x 5 members: 160 tiles of 16 rows).
 static int rows_plan(const lb_mlp* m, int n, bool train) {
   if (m->nh > 256) return 0;
-  if ((long)((n + 47) / 48) * m->K >= m->sms && rows_smem(m->nh, m->nout, 3, train) <= m->max_smem) return 3;
-  return rows_smem(m->nh, m->nout, 1, train) <= m->max_smem ? 1 : 0;
+  if ((long)((n + 47) / 48) * m->K >= m->dev.sms && rows_smem(m->nh, m->nout, 3, train) <= m->dev.max_smem) return 3;
+  return rows_smem(m->nh, m->nout, 1, train) <= m->dev.max_smem ? 1 : 0;
 }
 
 static RowsArgs rows_args(const lb_mlp* m, int n) {
@@ -1282,7 +1290,7 @@ static cudaError_t rows_train(lb_mlp* m, int rt, cudaStream_t s) {
   a.T = m->t;
   a.loss = m->loss;
   a.scale = 1.0f / ((float)m->n * (float)m->nout);
-  return launch_rows<true>(a, m->nh, rt, m->sms, s);
+  return launch_rows<true>(a, m->nh, rt, m->dev, s);
 }
 
 // Forward of every member on n rows of the inputs from row r0: outputs in m->y.
@@ -1290,8 +1298,8 @@ static cudaError_t rows_predict(lb_mlp* m, int rt, int r0, int n, cudaStream_t s
   RowsArgs a = rows_args(m, n);
   a.xf = m->xin + (long)r0 * m->nin;
   a.y = m->y + (long)r0 * m->nout;
-  if (rt == 3) return launch_predict(a, m->nh, m->sms, s);
-  return launch_rows<false>(a, m->nh, rt, m->sms, s);
+  if (rt == 3) return launch_predict(a, m->nh, m->dev, s);
+  return launch_rows<false>(a, m->nh, rt, m->dev, s);
 }
 
 // Rows of one part of a prediction on n rows.  Large results go to the host in up to kParts
@@ -1301,7 +1309,7 @@ static cudaError_t rows_predict(lb_mlp* m, int rt, int r0, int n, cudaStream_t s
 // part, so that no part ends in a wave of few.
 static int predict_part(const lb_mlp* m, int rt, int n) {
   if (rt != 3 || 8L * n * m->nout < (4L << 20)) return n;
-  const long slots = m->sms / m->K > 1 ? m->sms / m->K : 1, wave = 2 * 48 * slots;
+  const long slots = m->dev.sms / m->K > 1 ? m->dev.sms / m->K : 1, wave = 2 * 48 * slots;
   const long rows = ((n + wave - 1) / wave + kParts - 1) / kParts * wave;
   return rows < n ? (int)rows : n;
 }
@@ -1402,7 +1410,7 @@ static cudaError_t gemm_train(lb_mlp* m, cudaStream_t s) {
 // then reads 54 MB of partials; one member alone (24 tiles) needs the splits to fill the SMs.
 static int wgrad_parts(const lb_mlp* m, int ks) {
   const long h = m->nh / TM, o = (m->nout + TM - 1) / TM;
-  return ks <= 4 || 4 * (h * h + h * o + h) * m->K >= 3 * m->sms ? 1 : ks;
+  return ks <= 4 || 4 * (h * h + h * o + h) * m->K >= 3 * m->dev.sms ? 1 : ks;
 }
 
 // forward, loss and the gradients' partials of every member on the loaded data (sc:
@@ -1500,8 +1508,7 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
     lb_mlp_destroy(m);
     return merr(NULL, "device query failed: %s", cudaGetErrorString(ea)), LB_ERR_CUDA;
   }
-  m->sms = sms;
-  m->max_smem = (size_t)optin;
+  m->dev = RowsDevice{sms, (size_t)optin};
   for (cudaEvent_t& ev : m->done)
     if ((ea = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming)) != cudaSuccess) {
       lb_mlp_destroy(m);
