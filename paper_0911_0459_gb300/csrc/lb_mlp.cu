@@ -1572,6 +1572,7 @@ lb_status lb_mlp_create(int nin, int nh, int nout, int members, int max_batch, u
 void lb_mlp_destroy(lb_mlp* m) {
   if (!m) return;
   cudaStreamSynchronize(m->stream);
+  if (m->cap) cudaStreamSynchronize(m->cap);
   if (m->gexec) cudaGraphExecDestroy(m->gexec);
   for (void* p : m->owned) {
     if (m->have_alloc)
@@ -1664,9 +1665,7 @@ lb_status lb_mlp_train(lb_mlp* m, int steps, float lr, float lr_min, float wd, f
   return LB_OK;
 }
 
-lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* sd, float* members) {
-  if (!m || n < 1 || !x || !mean || !sd) return LB_ERR_ARG;
-  if (n > m->maxb) return merr(m, "batch larger than max_batch"), LB_ERR_ARG;
+static lb_status predict(lb_mlp* m, int n, const float* x, float* mean, float* sd, float* members) {
   MCK(cudaMemcpyAsync(m->xin, x, (size_t)n * m->nin * 4, cudaMemcpyHostToDevice, m->stream));
   const int rt = rows_plan(m, n, false), part = predict_part(m, rt, n);
   const long O = m->nout;
@@ -1699,6 +1698,17 @@ lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* s
   }
   MCK(cudaStreamSynchronize(s));  // (the copies follow the last kernels)
   return LB_OK;
+}
+
+lb_status lb_mlp_predict(lb_mlp* m, int n, const float* x, float* mean, float* sd, float* members) {
+  if (!m || n < 1 || !x || !mean || !sd) return LB_ERR_ARG;
+  if (n > m->maxb) return merr(m, "batch larger than max_batch"), LB_ERR_ARG;
+  const lb_status st = predict(m, n, x, mean, sd, members);
+  if (st != LB_OK) {  // no copy into the caller's arrays outlives the call
+    cudaStreamSynchronize(m->stream);
+    cudaStreamSynchronize(m->cap);
+  }
+  return st;
 }
 
 const char* lb_mlp_last_error(const lb_mlp* m) { return m ? m->err : g_mlp_err; }
