@@ -284,8 +284,8 @@ lb_status lb_set_kernel(lb_ctx *ctx, int variant);
 /* The kernel variant in use (1, 2, 3 or 4; automatic selection resolved). */
 lb_status lb_get_kernel(const lb_ctx *ctx, int *variant);
 
-/* Time each candidate kernel variant and tile on this lattice (the state is
- * saved and restored) and keep the fastest.  Returns the choice and its time per step in
+/* Time each candidate kernel variant and tile on this lattice, and those in use
+ * (the state is saved and restored), and keep the fastest.  Returns the choice and its time per step in
  * microseconds.  Waits for the stream. */
 lb_status lb_autotune(lb_ctx *ctx, int *tile_x, int *tile_y, double *us_per_step);
 
