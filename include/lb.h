@@ -271,7 +271,9 @@ lb_status lb_set_tile(lb_ctx *ctx, int tile_x, int tile_y);
 lb_status lb_get_tile(const lb_ctx *ctx, int *tile_x, int *tile_y);
 
 /* Choose the step kernel: 0 = automatic (the staged kernel where it fits and the
- * lattice is not small, else the sliding-window kernel), 1 = sliding-window kernel
+ * lattice is not small, else the sliding-window kernel; in the block storages the
+ * tile decides as well, tall bands on small lattices running staged, so that
+ * lb_set_tile can change the kernel), 1 = sliding-window kernel
  * (rows held in registers), 2 = staged kernel (rows brought into shared memory by bulk
  * copies; fits when nx % 8 == 0 and nx * ny <= 477218588, and at any nx for
  * the block storages, else LB_ERR_ARG)

@@ -142,6 +142,29 @@ static bool auto_staged(const lb_ctx* c) {
   return c->fluid > strips || c->fluid < least;
 }
 
+// The kernel in use.  On a lattice that auto_staged leaves to the sliding-window variant, a
+// tile that lb_set_tile brings (one found for the staged kernel, say) may have bands for
+// which the staged kernel is the faster one all the same: its ring hides the loads of a long
+// band and takes a row of blocks as one copy.  That holds for FP16 blocks at any height and
+// FP32 blocks above 16 rows where rows start on block boundaries (nx % 32 == 0), and for
+// FP16 blocks above two rows where they don't.  Us per step, strips and staged:
+//   FP16 blocks 1024 x 64   64 x 1: 4.0, 3.8;  128 x 1: 3.9, 4.1;  64 x 2: 4.6, 4.0;  128 x 16: 18.7, 13.2
+//               1536 x 60   128 x 1: 5.6, 4.2;  64 x 2: 4.9, 4.7
+//               1800 x 64   64 x 2: 5.5, 5.3;  128 x 2: 5.4, 6.1;  64 x 4: 7.5, 5.9;  128 x 16: 20.2, 14.5
+//   FP32 blocks 1024 x 64   128 x 8: 7.7, 7.6;  128 x 16: 13.8, 13.3;  64 x 32: 25.6, 23.0
+//               1800 x 64   64 x 8: 7.7, 9.4;  64 x 16: 13.7, 14.2;  128 x 32: 26.1, 27.2
+//   FP32 planes 1024 x 64   128 x 1: 3.9, 6.6;  128 x 32: 25.2, 49.3;  FP16 planes 128 x 32: 41.5, 48.2
+// In FP64 the two are within a tenth of each other up to 16 rows (liquid-gas 1024 x 64: 64 x 4
+// 21.2, 26.0;  64 x 16 65.8, 63.2).  The default tiles of small lattices in FP16 blocks run
+// staged by this, from 64 x 1 (1024 x 64: 3.98 -> 3.78) to 64 x 2.
+static bool staged_now(const lb_ctx* c) {
+  if (c->kernel != 0) return c->kernel == 2;
+  if (auto_staged(c)) return true;
+  const bool aligned = c->grid.nx % 32 == 0;
+  if (c->prm.storage == LB_STORAGE_F16_BLOCKED) return c->tile_y > (aligned ? 0 : 2);
+  return c->prm.storage == LB_STORAGE_F32_BLOCKED && aligned && c->tile_y > 16;
+}
+
 static OpArgs base_args(const lb_ctx* c) {
   OpArgs a;
   memset(&a, 0, sizeof a);
@@ -160,7 +183,7 @@ static OpArgs base_args(const lb_ctx* c) {
   a.thr = p.model == LB_MODEL_LIQUID_GAS ? 0.5 * (p.rho_l + p.rho_g) : 0.0;
   a.bx = c->tile_x;
   a.yc = c->tile_y;
-  a.staged = c->kernel == 2 || (c->kernel == 0 && auto_staged(c));
+  a.staged = staged_now(c);
   a.deep = c->deep;
   a.err = c->errflag;
   return a;
@@ -748,7 +771,7 @@ lb_status lb_get_kernel(const lb_ctx* c, int* variant) {
     *variant = 4;
     return LB_OK;
   }
-  const int k = c->kernel == 0 ? (auto_staged(c) ? 2 : 1) : c->kernel;
+  const int k = staged_now(c) ? 2 : 1;
   *variant = k == 2 && c->deep ? 3 : k;
   return LB_OK;
 }

@@ -1,0 +1,33 @@
+"""The step kernel behind the automatic choice, by lattice and tile, without a GPU (fake_cudart.cpp)."""
+from fake_cuda import run
+
+
+def test_tall_bands_on_small_block_lattices_run_the_staged_kernel(tmp_path):
+    """A tile given to a small lattice under the automatic choice.  In the block storages the
+    bands for which the staged kernel is faster run staged: FP16 at any height where rows start
+    on block boundaries and above two rows where they don't, FP32 above 16 rows on block
+    boundaries.  Other storages keep the sliding window at every height.  lb_get_kernel tells
+    what is launched."""
+    seen = run(tmp_path, r'''
+seen = []
+for nx in (1024, 1000, 612):
+    for st in (lb.STORAGE_F64, lb.STORAGE_F32, lb.STORAGE_F16DEV, lb.STORAGE_F32_BLOCKED, lb.STORAGE_F16_BLOCKED):
+        h = lattice(nx, 64, W.LG if st == lb.STORAGE_F64 else W.BINARY, st)
+        for t in [None] + [(x, y) for x in (64, 128, 256) for y in (1, 2, 3, 16, 17, 64)]:
+            if t: assert L.lb_set_tile(h, *t) == 0
+            log()
+            assert L.lb_step(h, 1) == 0
+            names = [n for _, _, n in launches("_kernel")]
+            assert len(names) == 1
+            seen.append([nx, st, tile(h)[1], kernel(h), "step_tma_kernel" in names[0]])
+        L.lb_destroy(h)
+print(json.dumps(seen))
+''')
+    for nx, st, ty, kernel, staged in seen:
+        assert kernel == (2 if staged else 1)
+        aligned = nx % 32 == 0
+        if st == 7:  # FP16 blocks (612 x 64: fewer than 40000 fluid nodes, staged at every tile)
+            expect = nx == 612 or ty > (0 if aligned else 2)
+        else:
+            expect = st == 6 and aligned and ty > 16
+        assert staged == expect, (nx, st, ty)
