@@ -63,12 +63,31 @@ static cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned bloc
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
-// The sliding-window variant runs as warp strips (step_strip).  In FP64 only bands of one
+// The sliding-window variant runs as warp strips (step_strip), but for the two cases below
+// and lattices beyond the strips' 32-bit offsets.  In FP64 only bands of one
 // or two rows do: there the FP64 pipe is the bound and the strips' 32 lanes for 30 columns
 // cost more than the window's barriers on lattices that fill the GPU (liquid-gas, us per
 // step: 256 x 32 at one row 8.5 -> 7.0, 4097 x 128 at two rows 123.1 -> 122.3, at six
 // 118.4 -> 127.6).
 constexpr int kStripRowsF64 = 2;
+
+// A strip produces 30 columns where the shared window's warp produces 32, so at some sizes
+// the strips need a second wave of CTAs while the window fits in one (16 warps an SM): there
+// the planes run the window (binary us per step, strips -> window: 2304 x 128 FP32 at 128 x 4
+// 11.5 -> 10.0, at 64 x 4 11.6 -> 10.5, FP16 13.4 -> 11.1; 3000 x 100 and 1536 x 200 alike).
+// CTAs of 256 columns are so large that one more on some SMs counts as well (1024 x 64 at
+// 256 x 1: 5.1 -> 4.5; FP64 at 256 x 2: 42.2 -> 31.2).  The liquid-gas FP32 strips, which
+// hold half the values, keep the second wave cheap except in those (2304 x 128: 64 x 4 7.5,
+// window 8.5; 256 x 4 9.7, 8.2).
+template <int MODEL, class S, int BX>
+static bool window_fills_one_wave(const OpArgs& a) {
+  constexpr unsigned per = 16 / (BX / 32), cols = BX / 32 * kStripCols;
+  const unsigned sms = (unsigned)device_sm_count();
+  const unsigned strips = tiles_1d((a.nx + cols - 1) / cols, a.ny, a.yc), window = tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc);
+  if (window > per * sms) return false;
+  if (MODEL == MODEL_LG && !std::is_same<typename S::A, double>::value) return BX == 256 && strips > per * sms;
+  return strips > per * sms || (BX == 256 && (strips + sms - 1) / sms > (window + sms - 1) / sms);
+}
 
 template <int MODEL, class S, int BX>
 static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
@@ -81,7 +100,8 @@ static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
   k.yc = a.yc;
   if constexpr (!is_blocked<S>::value) {
     constexpr bool F64 = std::is_same<typename S::A, double>::value;
-    if (F64 ? a.yc > kStripRowsF64 : 9ull * a.nx * a.ny >= 1ull << 32)  // (FP32 strips: 32-bit offsets)
+    if ((F64 ? a.yc > kStripRowsF64 : 9ull * a.nx * a.ny >= 1ull << 32) ||  // (FP32 strips: 32-bit offsets)
+        window_fills_one_wave<MODEL, S, BX>(a))
       return launch_pdl(step_kernel<MODEL, S, BX>, tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc), BX, 0, s, k);
   }
   return launch_pdl(strip_kernel<MODEL, S, BX / 32>,

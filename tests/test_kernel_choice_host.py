@@ -31,3 +31,44 @@ print(json.dumps(seen))
         else:
             expect = st == 6 and aligned and ty > 16
         assert staged == expect, (nx, st, ty)
+
+
+def test_sliding_window_runs_the_kernel_whose_tiles_fit_in_one_wave(tmp_path):
+    """Strips of 30 columns against tiles of 32 a warp: where the tiles fit in one wave of 16
+    warps on each of the 152 SMs and the strips don't, the planes run the shared window."""
+    seen = run(tmp_path, r'''
+seen = []
+for nx, ny in ((1024, 64), (700, 40), (2304, 128), (1000, 200)):
+    for model, st in ((W.LG, lb.STORAGE_F64), (W.LG, lb.STORAGE_F32), (W.BINARY, lb.STORAGE_F64), (W.BINARY, lb.STORAGE_F32),
+                      (W.BINARY, lb.STORAGE_F16DEV), (W.BINARY, lb.STORAGE_F32_BLOCKED)):
+        h = lattice(nx, ny, model, st)
+        assert L.lb_set_kernel(h, 1) == 0
+        for t in [(x, y) for x in (64, 128, 256) for y in (1, 2, 3, 4, 8)]:
+            assert L.lb_set_tile(h, *t) == 0
+            log()
+            assert L.lb_step(h, 1) == 0
+            (grid, block, name), = launches("_kernel")
+            assert kernel(h) == 1 and block == t[0]
+            seen.append([nx, ny, model, st, t, grid, "strip_kernel" in name])
+        L.lb_destroy(h)
+print(json.dumps(seen))
+''')
+    windows = set()
+    for nx, ny, model, st, (tx, ty), grid, strip in seen:
+        bands = -(-ny // ty)
+        strips, window = -(-nx // (tx // 32 * 30)) * bands, -(-nx // tx) * bands
+        assert grid == (strips if strip else window)
+        wave = 152 * 16 // (tx // 32)
+        one = window <= wave < strips
+        if st == 6:
+            expect = True
+        elif model == 0 and st == 1:
+            expect = not (tx == 256 and one)
+        else:
+            expect = not (one or (tx == 256 and window <= wave and -(-strips // 152) > -(-window // 152)))
+            if st == 0 and ty > 2:
+                expect = False
+        assert strip == expect, (nx, ny, model, st, tx, ty)
+        if not strip:
+            windows.add((nx, tx, ty, st))
+    assert {(2304, 128, 4, 1), (2304, 64, 4, 2), (1024, 256, 2, 0)} <= windows
