@@ -68,6 +68,7 @@ struct lb_batch {
   int kernel;      // 0 automatic, 1 sliding-window body, 2 staged body
   int deep;        // staged body: the deeper of its two rings
   int staged_ok;   // every lattice fits the staged body (nx % 8 == 0, 9 nx ny < 2^32)
+  int many;        // staged body: the one for as many CTAs as fit (batch_has_many)
   int grid_blocks;
   unsigned int extra_arrivals;
   unsigned long long limit_ns;
@@ -245,17 +246,19 @@ static cudaError_t run_sliding(lb_batch* b, int nsteps, cudaStream_t s, int* per
   return cudaLaunchKernelEx(&cfg, batch_step_kernel<S, BX>, a);
 }
 
-template <class S, int BX, int NS>
+template <class S, int BX, int NS, bool MANY = false>
 static cudaError_t run_staged(lb_batch* b, int nsteps, cudaStream_t s, int* per) {
+  if constexpr (!MANY && batch_has_many<S, BX>())
+    if (b->many) return run_staged<S, BX, NS, true>(b, nsteps, s, per);
   using L = TmaLayout<MODEL_BINARY, S, BX, NS>;
   static bool configured = false;  // dynamic shared memory opt-in, once per process
   if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(batch_tma_kernel<S, BX, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(batch_tma_kernel<S, BX, NS, MANY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)L::BYTES);
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  if (per) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, batch_tma_kernel<S, BX, NS>, BX + 32, L::BYTES);
+  if (per) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per, batch_tma_kernel<S, BX, NS, MANY>, BX + 32, L::BYTES);
   BatchArgs<S> a;
   fill_args(b, nsteps, a);
   cudaLaunchConfig_t cfg = {};
@@ -268,7 +271,7 @@ static cudaError_t run_staged(lb_batch* b, int nsteps, cudaStream_t s, int* per)
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, batch_tma_kernel<S, BX, NS>, a);
+  return cudaLaunchKernelEx(&cfg, batch_tma_kernel<S, BX, NS, MANY>, a);
 }
 
 template <int NW>
@@ -359,8 +362,20 @@ static lb_status build_tiles(lb_batch* b) {
   int dev = 0, sms = 0, per = 0;
   BCK(cudaGetDevice(&dev));
   BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  b->many = 0;
   BCK(run_batch(b, 0, b->stream, &per));
   if (per < 1) return berr(b, "the persistent kernel does not fit on an SM"), LB_ERR_CUDA;
+  const long wave = (long)per * sms, nt = b->ntiles;
+  if (b->storage == LB_STORAGE_F16_BLOCKED && batch_variant(b) == 2 && b->tile_x < 256 && 10 * nt > 11 * wave &&
+      10 * nt <= 13 * wave) {
+    b->many = 1;
+    int most = 0;
+    BCK(run_batch(b, 0, b->stream, &most));
+    if ((long)most * sms >= nt)
+      per = most;
+    else
+      b->many = 0;
+  }
   const int blocks = std::max(1, std::min(per * sms, b->ntiles));
   // longest processing time first onto the least loaded CTA
   std::vector<int> order(tiles.size());

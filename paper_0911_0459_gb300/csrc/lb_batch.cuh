@@ -173,21 +173,32 @@ __device__ __forceinline__ bool grid_barrier_checked(GridBarrier* b, unsigned in
 //                6, 5, 4 (3: 34.8);  256: 34.7, 36.9 (deep ring) at 2, 1
 //   FP16 blocks  128 columns: 31.0, 46.5, 40.3 at 5, 3, 2 CTAs;  64: 25.3, 32.5, 35.4 at
 //                6, 5, 4 (3: 35.2);  256: 46.2, 49.0, 38.4 at 3, 2, 1
-template <class S, int BX, int NS>
+// A sweep whose tiles are a tenth to three tenths more than the resident CTAs waits for the
+// few CTAs that take two.  FP16 blocks at 64 and 128 columns have a second body for these,
+// compiled for five CTAs of 128 columns and as many of 64 as shared memory holds (MANY): the
+// tiles then fit in one wave, which is worth 100 to 150 bytes of spills a thread (run_sampled of 40 steps, us, few -> many CTAs: 8 capillaries,
+// 520 tiles of 128 x 8: 1059 -> 999; 10 capillaries, 694 tiles of 64 x 16: 1456 -> 1261; above
+// that 704 tiles of 128 x 4: 809, 829; below, 475 of 128 x 12: 1003, 1199).
+template <class S, int BX>
+constexpr bool batch_has_many() {
+  return std::is_same<S, SF16B>::value && BX < 256;
+}
+template <class S, int BX, int NS, bool MANY>
 constexpr int batch_min_blocks() {
   if constexpr (is_blocked<S>::value) {
     using L = TmaLayout<MODEL_BINARY, S, BX, NS>;
     constexpr bool F16 = std::is_same<S, SF16B>::value;
     constexpr int by_smem = int(233472 / (L::BYTES + 1024));
-    constexpr int few = BX == 64 ? 4 : (BX == 128 ? (F16 ? 3 : 2) : (F16 ? 2 : 1));
-    return by_smem < few ? (by_smem < 1 ? 1 : by_smem) : few;
+    constexpr int most = MANY      ? 65536 / ((BX + 32) * 80)
+                         : BX == 64 ? 4 : (BX == 128 ? (F16 ? 3 : 2) : (F16 ? 2 : 1));
+    return by_smem < most ? (by_smem < 1 ? 1 : by_smem) : most;
   } else {
     return tma_min_blocks_of<MODEL_BINARY, S, BX, NS>();
   }
 }
 
-template <class S, int BX, int NS>
-__global__ void __launch_bounds__(BX + 32, (batch_min_blocks<S, BX, NS>())) batch_tma_kernel(BatchArgs<S> a) {
+template <class S, int BX, int NS, bool MANY>
+__global__ void __launch_bounds__(BX + 32, (batch_min_blocks<S, BX, NS, MANY>())) batch_tma_kernel(BatchArgs<S> a) {
   extern __shared__ __align__(128) unsigned char smem[];
   const Ring<MODEL_BINARY, S, BX, NS> R = ring_init<MODEL_BINARY, S, BX, NS>(smem);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
