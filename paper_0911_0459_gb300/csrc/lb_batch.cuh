@@ -176,9 +176,10 @@ __device__ __forceinline__ bool grid_barrier_checked(GridBarrier* b, unsigned in
 // A sweep whose tiles are a tenth to three tenths more than the resident CTAs waits for the
 // few CTAs that take two.  FP16 blocks at 64 and 128 columns have a second body for these,
 // compiled for five CTAs of 128 columns and as many of 64 as shared memory holds (MANY): the
-// tiles then fit in one wave, which is worth 100 to 150 bytes of spills a thread (run_sampled of 40 steps, us, few -> many CTAs: 8 capillaries,
-// 520 tiles of 128 x 8: 1059 -> 999; 10 capillaries, 694 tiles of 64 x 16: 1456 -> 1261; above
-// that 704 tiles of 128 x 4: 809, 829; below, 475 of 128 x 12: 1003, 1199).
+// tiles then fit in one wave, which is worth 100 to 150 bytes of spills a thread (run_sampled
+// of 40 steps, us, few -> many CTAs: 8 capillaries, 520 tiles of 128 x 8: 1047 -> 965; 10
+// capillaries, 694 tiles of 64 x 16: 1456 -> 1283; outside that range the few are faster: 475
+// tiles of 128 x 12 1003, 1207; 704 of 128 x 4 805, 836; 674 of 128 x 8, the worst, 1155, 1115).
 template <class S, int BX>
 constexpr bool batch_has_many() {
   return std::is_same<S, SF16B>::value && BX < 256;
