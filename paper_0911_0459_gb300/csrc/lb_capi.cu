@@ -420,10 +420,9 @@ static void default_tile(lb_ctx* c) {
     per_sm = lg ? 4 : 2;
     most = 10;
   } else {
-    // planar storages: wide tiles, whose longer copies suit the copy engine, unless they
-    // leave SMs without a tile
-    bx = cols = (long)((nx + 255) / 256) * ny < device_sm_count() ? 128 : 256;
-    per_sm = bx == 256 ? 3 : 5;
+    // planar storages: wide tiles, whose longer copies suit the copy engine
+    bx = cols = 256;
+    per_sm = 3;
     most = lg ? 16 : (st == LB_STORAGE_F16DEV ? 12 : 8);
   }
   while (bx > 64 && nx <= bx / 2) {  // a narrow lattice: no idle half tiles

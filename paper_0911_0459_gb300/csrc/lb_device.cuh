@@ -324,7 +324,6 @@ struct SF32B {
   static constexpr int kGOff = 1;          // g_i is the element after f_i
   static constexpr int kG0 = 0;            // (g_0 pairs with f_0)
   __device__ static size_t at(size_t n, int i) { return (n >> 5) * kBlock + 64 * i + 2 * (n & 31); }
-  __device__ static uint32_t at32(uint32_t n, int i) { return (n >> 5) * kBlock + 64 * i + 2 * (n & 31); }
   // elements of a state of N nodes (the last block padded)
   __device__ static unsigned long long lim(unsigned long long N) { return 18ull * ((N + 31) & ~31ull); }
   // shared-memory stage of whole blocks: stage column c lies in block c / 32
@@ -369,15 +368,6 @@ struct SF32B {
     LB_GUARD(at(n, i), lim(N) - 1, A(0));
     return __ldcg(g + at(n, i));
   }
-  // 32-bit element offsets (needs 18 * 32 * ceil(N / 32) < 2^32)
-  __device__ static void sfo(T* __restrict__ f, uint32_t N, uint32_t n, int i, A v, const Rest&) {
-    LB_GUARD(at32(n, i), lim(N), );
-    f[at32(n, i)] = v;
-  }
-  __device__ static void sgo(T* __restrict__ g, float* __restrict__, uint32_t N, uint32_t n, int i, A v) {
-    LB_GUARD(at32(n, i), lim(N) - 1, );
-    g[at32(n, i)] = v;
-  }
   __device__ static void zf(T* __restrict__ f, size_t N, size_t n, int i) {
     LB_GUARD(at(n, i), lim(N), );
     f[at(n, i)] = 0.0f;
@@ -404,7 +394,6 @@ struct SF16B {
   static constexpr int kG0Stride = 304;    // floats per block
   __device__ static int off(int r, int i) { return i == 0 ? r : 32 + 64 * (i - 1) + 2 * r; }
   __device__ static size_t at(size_t n, int i) { return (n >> 5) * kBlock + off((int)(n & 31), i); }
-  __device__ static uint32_t at32(uint32_t n, int i) { return (n >> 5) * kBlock + off((int)(n & 31), i); }
   __device__ static size_t at0(size_t n) { return (n >> 5) * kG0Stride + (n & 31); }
   // halves of a state of N nodes (the last block padded)
   __device__ static unsigned long long lim(unsigned long long N) { return 19ull * ((N + 31) & ~31ull); }
@@ -485,25 +474,6 @@ struct SF16B {
     }
     LB_GUARD(at(n, i), lim(N) - kGOff, );
     g[at(n, i)] = __float2half_rn(v);
-  }
-  // 32-bit element offsets (needs 19 * 32 * ceil(N / 32) < 2^32)
-  __device__ static void sfo(T* __restrict__ f, uint32_t N, uint32_t n, int i, A v, const Rest& r) {
-    LB_GUARD(at32(n, i), lim(N), );
-    f[at32(n, i)] = __float2half_rn(v - rest_w(r, i));
-  }
-  __device__ static void sfor(T* __restrict__ f, uint32_t N, uint32_t n, int i, A v) {
-    LB_GUARD(at32(n, i), lim(N), );
-    f[at32(n, i)] = __float2half_rn(v);
-  }
-  __device__ static void sgo(T* __restrict__ g, float* __restrict__ g0, uint32_t N, uint32_t n, int i, A v) {
-    if (i == 0) {
-      const uint32_t o = (n >> 5) * kG0Stride + (n & 31);
-      LB_GUARD(o, lim0(N), );
-      g0[o] = v;
-      return;
-    }
-    LB_GUARD(at32(n, i), lim(N) - kGOff, );
-    g[at32(n, i)] = __float2half_rn(v);
   }
   __device__ static void zf(T* __restrict__ f, size_t N, size_t n, int i) {
     LB_GUARD(at(n, i), lim(N), );

@@ -45,7 +45,7 @@ constexpr int kGraphSteps = 16;  // training steps per captured graph: the gap b
 constexpr int kParts = 4;  // of a large prediction
 constexpr int kBiasGroups = 8;  // partial sums of a bias gradient (32 row classes each)
 
-enum { EPI_BIAS_F32 = 0, EPI_BIAS_TANH = 1, EPI_LOSS = 2, EPI_DTANH = 3, EPI_PART = 4 };
+enum { EPI_BIAS_F32 = 0, EPI_BIAS_TANH = 1, EPI_LOSS = 2, EPI_DTANH = 3 };
 
 // C (M x N) = A B over K rows [kb, ke).  Non-transposed operands hold K contiguous
 // (A[m][k], B[n][k]), transposed ones hold the other index contiguous (A[k][m],
@@ -122,13 +122,13 @@ __device__ __forceinline__ void cp_wait() {
 // phase reads lie in different banks.
 __device__ __forceinline__ uint32_t swz(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
 
-// One operand of the ring: 64 x 64 values a stage, 16-byte chunks of NTH threads (rows
-// tid / 8 + NTH / 8 i, chunk tid % 8).  Not transposed: rows are the output index (from r0,
+// One operand of the ring: 64 x 64 values a stage, 16-byte chunks of 128 threads (rows
+// tid / 8 + 16 i, chunk tid % 8).  Not transposed: rows are the output index (from r0,
 // below rmax), columns K (a multiple of 8 ends the array).  Transposed: rows K, columns
 // the output index.  What a thread can know beforehand is kept here.
-template <bool TRANS, int NTH>
+template <bool TRANS>
 struct Operand {
-  static constexpr int kRows = NTH / 8, kChunks = 64 / kRows;
+  static constexpr int kRows = 16, kChunks = 64 / kRows;
   const bf16* p;   // this thread's first chunk of the next stage
   long step, row;  // elements to the next stage, and to the thread's next row
   uint32_t dst;    // its place in a stage
@@ -162,17 +162,17 @@ struct Operand {
   }
 };
 
-// The 64x64 tile (m0, n0) of member mem, K rows [kb, ke), in the accumulators of
-// 2 WN warps (warp w: rows 32 (w / WN), 64 / WN columns from 64 / WN (w % WN)).  SPLIT: every kc rows the
+// The 64x64 tile (m0, n0) of member mem, K rows [kb, ke), in the accumulators of four
+// warps (warp w: rows from 32 (w / 2), columns from 32 (w % 2)).  SPLIT: every kc rows the
 // accumulators are added to a running sum and start again from zero (kc a multiple of
 // 16 unless it covers the range).
-template <bool TA, bool TB, int WN = 2, int ST = kStages, bool SPLIT = false>
+template <bool TA, bool TB, int ST = kStages, bool SPLIT = false>
 __device__ __forceinline__ void gemm_tile(const bf16* A, long lda, int M, const bf16* B, long ldb, int bmax, int m0,
-                                          int n0, int kb, int ke, unsigned char* smem, float acc[2][8 / WN][4],
+                                          int n0, int kb, int ke, unsigned char* smem, float acc[2][4][4],
                                           int kc = 0) {
-  constexpr int NI = 8 / WN, NTH = 64 * WN;
+  constexpr int NI = 4;  // fragments of 8 columns per warp
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int wm = (warp / WN) * 32, wn = (warp % WN) * (8 * NI);
+  const int wm = (warp / 2) * 32, wn = (warp % 2) * 32;
   const uint32_t sb = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
 #pragma unroll
   for (int i = 0; i < 2; ++i)
@@ -181,8 +181,8 @@ __device__ __forceinline__ void gemm_tile(const bf16* A, long lda, int M, const 
 #pragma unroll
       for (int k = 0; k < 4; ++k) acc[i][j][k] = 0.0f;
   const int nk = (ke - kb + TK - 1) / TK;
-  Operand<TA, NTH> oa(A, lda, m0, M, kb);
-  Operand<TB, NTH> ob(B, ldb, n0, bmax, kb);
+  Operand<TA> oa(A, lda, m0, M, kb);
+  Operand<TB> ob(B, ldb, n0, bmax, kb);
   uint32_t wr = sb, rd = sb;  // the stages written and read next
   auto load = [&](int c) {
     if (c < nk) {
@@ -273,11 +273,11 @@ __device__ __forceinline__ void gemm_tile(const bf16* A, long lda, int M, const 
 
 // Store of the accumulators: f(m, n, v0, v1) for every pair of neighbouring columns
 // n, n + 1 inside the output (N is even, so a pair is inside as a whole).
-template <int WN = 2, class F>
-__device__ __forceinline__ void for_pairs(const float acc[2][8 / WN][4], int m0, int n0, int M, int N, F f) {
-  constexpr int NI = 8 / WN;
+template <class F>
+__device__ __forceinline__ void for_pairs(const float acc[2][4][4], int m0, int n0, int M, int N, F f) {
+  constexpr int NI = 4;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int wm = (warp / WN) * 32, wn = (warp % WN) * (8 * NI);
+  const int wm = (warp / 2) * 32, wn = (warp % 2) * 32;
   const int gq = lane >> 2, tq = lane & 3;
 #pragma unroll
   for (int mi = 0; mi < 2; ++mi)
@@ -988,11 +988,11 @@ __global__ void __launch_bounds__(kWgradThreads) wgrad_kernel(WgradArgs a) {
         const int m0 = t / a.ntn[q] * TM, n0 = t % a.ntn[q] * TN;
         const int kb = y * a.kc, ke = a.parts == 1 ? g.K : min(g.K, kb + a.kc);
         float acc[2][4][4];
-        gemm_tile<true, true, 2, kWgradStages, true>(g.A + mem * g.a_mem, g.lda, g.M, g.B + mem * g.b_mem, g.ldb, g.b_cols,
+        gemm_tile<true, true, kWgradStages, true>(g.A + mem * g.a_mem, g.lda, g.M, g.B + mem * g.b_mem, g.ldb, g.b_cols,
                                                   m0, n0, kb, ke, smem, acc, a.kc);
         float* C = g.Cf + ((long)mem * a.parts + y) * g.cf_mem;
         const int N = g.N;
-        for_pairs<2>(acc, m0, n0, g.M, (N + 1) & ~1, [&](int m, int n, float v0, float v1) {
+        for_pairs(acc, m0, n0, g.M, (N + 1) & ~1, [&](int m, int n, float v0, float v1) {
           float* o = C + (long)m * N + n;
           if (!(N & 1)) {
             *reinterpret_cast<float2*>(o) = make_float2(v0, v1);
@@ -1213,7 +1213,6 @@ struct lb_mlp {
   float *xin, *mean, *sd;
   cudaEvent_t done[kParts];  // the parts of a prediction
   cudaGraphExec_t gexec;
-  int graph_n;
   char err[512];
 };
 
