@@ -121,15 +121,27 @@ static bool staged_ok(int storage, int nx, int ny) {
   return storage == LB_STORAGE_F32_BLOCKED || storage == LB_STORAGE_F16_BLOCKED || staged_fits(nx, ny);
 }
 
-// The automatic kernel: staged where it fits, except on small lattices, where the warp
-// strips of the sliding-window variant have the shorter chain of latencies.  The planar
-// storages' rings (18 copies a row) take longest to fill; us per step, staged -> strips:
-// 704 x 40 FP32 6.1 -> 2.8, 2048 x 64 7.4 -> 5.7, 1000 x 200 9.6 -> 7.8, 4096 x 128 14.6 ->
-// 15.0; liquid-gas FP64 256 x 32 9.0 -> 7.0, 1000 x 200 61.6 -> 55.2, 4096 x 128 118 -> 122;
-// binary FP64 1024 x 64 37.3 -> 34.7, 2048 x 64 52.9 -> 62.1; FP32 blocks (one copy a row)
-// 704 x 40 3.2 -> 2.6, 1024 x 64 4.2 -> 3.5, 2048 x 64 5.6 -> 5.3, 1000 x 200 7.2 -> 7.1, 4096 x
-// 128 11.2 -> 13.8; FP16 blocks 704 x 40 3.2 -> 3.4, 1024 x 64 4.2 -> 3.7, 2048 x 64 5.5 -> 5.3,
-// 1000 x 200 6.7 -> 7.2.
+// The automatic kernel by the lattice alone: staged where it fits, except on small lattices,
+// where the warp strips of the sliding-window variant have the shorter chain of latencies (the
+// planar storages' rings, 18 copies a row, take longest to fill).  Us per step on lattices that
+// are half tube, best tile of each, staged -> sliding window:
+//   FP32 planes  704 x 40 6.2 -> 2.7;  2048 x 64 8.4 -> 5.3;  1000 x 200 9.5 -> 7.4;  2304 x 128 12.3 ->
+//                10.0;  4096 x 96 14.2 -> 12.4;  4096 x 128 16.5 -> 15.6 (the ring keeps its rate
+//                beyond: 16384 x 256 88.4 -> 101)
+//   FP16 planes  704 x 40 6.2 -> 3.7;  1000 x 200 9.3 -> 8.0;  2304 x 128 12.0 -> 11.1;  4096 x 96 13.6 -> 13.4;
+//                4096 x 128 15.7 -> 16.9;  liquid-gas FP32  704 x 40 4.4 -> 2.3;  1000 x 200 6.9 -> 5.4;
+//                2304 x 128 8.8 -> 7.5;  4096 x 128 11.6 -> 10.4
+//   FP32 blocks  704 x 40 3.1 -> 2.6;  1024 x 64 4.1 -> 3.6;  2048 x 64 5.5 -> 5.2;  1000 x 200 7.2 -> 7.1;
+//                4096 x 64 7.9 -> 8.3;  4096 x 128 12.5 -> 14.6
+//   FP16 blocks  704 x 40 3.1 -> 3.4;  1024 x 64 3.8 -> 3.9;  2048 x 64 5.0 -> 5.3;  1000 x 200 7.1 -> 8.5
+//                (between the lines the tile decides: staged_now)
+//   FP64         liquid-gas 256 x 32 9.7 -> 5.8;  1000 x 200 54.4 -> 48.2;  4096 x 64 64.9 -> 59.5;  4096 x 128
+//                110.5 -> 107.6;  binary 1024 x 64 38.0 -> 28.5;  2048 x 64 63.2 -> 54.7;  4096 x 64 104.3 ->
+//                103.8;  4096 x 128 192 -> 190
+// The FP64 lines (250000 and 70000 nodes) were drawn with the collision before its row
+// summaries, when the staged kernel won above them (binary 2048 x 64 52.9 against 62.1 on
+// 102000 nodes); with the collision as it is the two are closer than a tenth from 256000
+// nodes on, and below that the line for the binary model could lie higher.
 static bool auto_staged(const lb_ctx* c) {
   if (!staged_ok(c->prm.storage, c->grid.nx, c->grid.ny)) return false;
   long strips, least = 0;  // largest and smallest number of fluid nodes that runs as strips
@@ -371,14 +383,15 @@ static lb_status default_state(lb_ctx* c) {
 // lattices of many waves.  A small lattice with the bands of a large one leaves most
 // SMs idle (256 x 32 FP64 at 128 x 16 is four CTAs); bands of one row recompute the
 // sums of two halo rows for each row, which no longer pays once a wave is full.
-// Measured in us per step, 128 x 16 for every lattice against this rule:
-//   256 x 32 liquid-gas FP64      84.0   7.0 (64 x 1)
-//   700 x 40 FP32 planes          15.8   2.8 (64 x 1)
-//   2048 x 64 FP32 planes         27.1   5.7 (64 x 2)       FP32 blocks  13.6   5.3 (64 x 2)
-//   4096 x 128 FP32 blocks        17.6  11.2 (128 x 6)      moments      15.0  11.3 (128 x 6)
-//   16384 x 256 FP32 blocks       85.4  79.6 (128 x 8)      moments      50.5  48.2 (128 x 12)
-//   16384 x 256 FP32 planes       97.0  90.5 (256 x 8)      FP64         888   662 (64 x 10)
-//   (the liquid-gas FP64 figures with the collision as it is now; 128 x 16 before it)
+// Us per step, 128 x 16 in the staged kernel for every lattice (as it was) against this rule:
+//   256 x 32 liquid-gas FP64      84.0   5.9 (64 x 1)
+//   700 x 40 FP32 planes          15.8   2.7 (64 x 1)
+//   2048 x 64 FP32 planes         27.1   5.6 (64 x 2)       FP32 blocks  13.6   5.3 (64 x 2)
+//   4096 x 128 FP32 blocks        17.6  11.3 (128 x 6)      moments      15.0  10.9 (128 x 6)
+//   16384 x 256 FP32 blocks       85.4  77.2 (128 x 8)      moments      50.5  48.0 (128 x 12)
+//   16384 x 256 FP32 planes       97.0  88.4 (256 x 8)      liquid-gas FP64  888   644 (64 x 10)
+//   (the FP64 figures on the left with the collision before its row summaries; with the one in
+//   use 16384 x 256 takes 704 at 128 x 16)
 static void default_tile(lb_ctx* c) {
   const int nx = c->grid.nx, ny = c->grid.ny, st = c->prm.storage;
   const bool lg = c->prm.model == LB_MODEL_LIQUID_GAS;

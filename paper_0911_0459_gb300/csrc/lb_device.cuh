@@ -2,10 +2,13 @@
 // collision + streaming + walls) for sm_103a.
 //
 // Layout: structure of arrays, plane i of f at f + i*N (N = nx*ny), node (x, y)
-// at y*nx + x.  A CTA owns BX consecutive columns and a band of rows; it walks
-// up the band with a 4-slot ring of rho/phi rows in shared memory (the 3x3
-// stencils of Eq. (best) need rows y-1, y, y+1) while the populations of the
-// next two rows are already in flight in registers.  Post-collision populations
+// at y*nx + x, or blocks of 32 nodes (SF32B, SF16B).  The sliding-window variant
+// here walks up a band of rows while the populations of the next two rows are
+// already in flight in registers (the 3x3 stencils of Eq. (best) need the densities
+// of rows y-1, y, y+1): as strips of 30 columns, one per warp, which take the
+// neighbouring columns by shuffles (step_strip), or, where those do not apply or
+// serve (lb_ops_impl.cuh), as a CTA of BX columns with a 4-slot ring of rho/phi
+// rows in shared memory (step_band).  Post-collision populations
 // are pushed to r + e_i in the other buffer; a push into a solid node returns
 // to the source node in the opposite direction (bounce-back, Sec. 2.2).  The
 // stored state is the post-streaming state before the boundary-node rest rule;
@@ -1356,7 +1359,7 @@ __device__ __forceinline__ void step_band(const Geom& G, const Phys<typename S::
 // the two idle lanes cost less than the barriers in FP32.  Us per step, shared window ->
 // strips, best tile of each: 704 x 40 FP32 planes 3.68 -> 2.76, 2048 x 64 6.43 -> 5.58,
 // 1000 x 200 8.14 -> 7.79, 16391 x 256 104.4 -> 101.3; 256 x 32 liquid-gas FP64 8.5 ->
-// 7.0 (its FP64 sums without the halo columns).  FP32 and FP16 planes are addressed by 32-bit
+// 7.0 (its FP64 sums without the halo columns; 5.9 with the collision as it is now).  FP32 and FP16 planes are addressed by 32-bit
 // element offsets (planes of 9 N >= 2^32 values take the shared window): 700 x 40 2.85 ->
 // 2.81, 2048 x 64 5.77 -> 5.66; the FP64 strips spilled with them.
 constexpr int kStripCols = 30;

@@ -431,7 +431,7 @@ struct RowsArgs {
   float scale;
 };
 
-constexpr int kRowThreads = 256;  // eight warps (sixteen of half the columns: 49 instead of 47 us)
+constexpr int kRowThreads = 256;  // eight warps (sixteen of half the columns: 49 instead of 46 us)
 
 // Shared memory of a row-tile CTA in bytes (o16: n_out rounded up to 16).
 constexpr size_t rows_smem(int nh, int nout, int rt, bool train) {
@@ -1405,7 +1405,7 @@ static cudaError_t gemm_train(lb_mlp* m, cudaStream_t s) {
 
 // Parts the weight gradients are left in: 1 where the tiles fill three quarters of the
 // SMs, or where a CTA's pass over all rows is short, else one per split.  4096 rows x 5
-// members (120 tiles): 38 us in one part, 41 us in 32 parts and 2 us more in AdamW, which
+// members (120 tiles): 33 us in one part, 39 us in 32 parts and 2 us more in AdamW, which
 // then reads 54 MB of partials; one member alone (24 tiles) needs the splits to fill the SMs.
 static int wgrad_parts(const lb_mlp* m, int ks) {
   const long h = m->nh / TM, o = (m->nout + TM - 1) / TM;

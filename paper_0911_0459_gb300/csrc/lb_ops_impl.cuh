@@ -65,10 +65,14 @@ static cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned bloc
 
 // The sliding-window variant runs as warp strips (step_strip), but for the two cases below
 // and lattices beyond the strips' 32-bit offsets.  In FP64 only bands of one
-// or two rows do: there the FP64 pipe is the bound and the strips' 32 lanes for 30 columns
-// cost more than the window's barriers on lattices that fill the GPU (liquid-gas, us per
-// step: 256 x 32 at one row 8.5 -> 7.0, 4097 x 128 at two rows 123.1 -> 122.3, at six
-// 118.4 -> 127.6).
+// or two rows do.  The strips form the row summaries of all three rows anew for every node,
+// the window does too, and the strips' 32 lanes for 30 columns stand against its barriers: us
+// per step, window -> strips, liquid-gas 1024 x 64 at two rows 19.5 -> 17.5, 1000 x 200 50.2 ->
+// 48.4; 4096 x 128 at three rows 107.6 -> 113.9 (128 columns), at four 109.4 -> 115.9, at six
+// 117.6 -> 110.6 (64 columns); binary 4096 x 128 at three 190.0 -> 194.5, at four 193.1 -> 199.8,
+// 4097 x 128 at six 231.7 -> 191.8; liquid-gas 256 x 32 at four 19.9 -> 17.1.  Above two rows the
+// best tiles on 4096 x 128 are the window's (107.6 and 190.0 against 110.6 and 191.8); on small
+// lattices, and on wide ones at six rows, the strips would be faster.
 constexpr int kStripRowsF64 = 2;
 
 // A strip produces 30 columns where the shared window's warp produces 32, so at some sizes
