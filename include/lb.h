@@ -265,7 +265,9 @@ long lb_time(const lb_ctx *ctx);
 long lb_fluid_nodes(const lb_ctx *ctx);
 
 /* Choose the tile of the step kernel: tile_x threads per block along x (64,
- * 128 or 256) and tile_y rows per block (1 .. ny).  Invalidates the captured
+ * 128 or 256) and tile_y rows per block (1 .. ny).  The automatic kernel goes by the
+ * lattice and, in the block storages, by the tile: to restore a tuned or saved choice, set its
+ * kernel (lb_get_kernel, lb_set_kernel) as well as its tile.  Invalidates the captured
  * step graph. */
 lb_status lb_set_tile(lb_ctx *ctx, int tile_x, int tile_y);
 lb_status lb_get_tile(const lb_ctx *ctx, int *tile_x, int *tile_y);
