@@ -112,6 +112,28 @@ static cudaError_t launch_step(const OpArgs& a, cudaStream_t s) {
                     tiles_1d((a.nx + BX / 32 * kStripCols - 1) / (BX / 32 * kStripCols), a.ny, a.yc), BX, 0, s, k);
 }
 
+// When a CTA of the staged kernel lets the next step's CTAs in: as soon as its last row is
+// on its way, which hides most of their start, or only when it ends.  With CTAs that are few
+// and long the former puts the next step where this one ends first, several CTAs on one SM and
+// none on another.  That costs FP64 bands of six rows and more and the block storages' (from
+// three rows in FP32, from six in FP16) up to half a step while the CTAs are between half of
+// one and about six tenths of the resident ones an SM; beyond, and in bands of fewer rows and
+// the planes, whose copies set the pace, letting them in early is the faster way or makes no
+// difference.  Us per step, early -> at the end:
+//   FP64         1000 x 200 binary 64 x 12 130.3 -> 85.1, liquid-gas 128 x 8 93.1 -> 65.7;  4096 x 128
+//                liquid-gas 64 x 32 168.7 -> 123.9;  1000 x 200 binary 128 x 8 102.3 -> 109.6 (the worst)
+//   FP32 blocks  1000 x 200 64 x 6 10.3 -> 8.3;  2304 x 128 128 x 8 11.5 -> 9.3;  704 x 40 128 x 3 4.1 -> 4.4
+//   FP16 blocks  4096 x 128 128 x 10 13.9 -> 11.6;  2304 x 128 128 x 6 9.8 -> 8.5;  1536 x 60 128 x 6 6.4 -> 6.8
+template <class S, int BX>
+static bool early_trigger(const OpArgs& a, unsigned grid) {
+  constexpr bool F64 = std::is_same<typename S::A, double>::value;
+  if (!F64 && !is_blocked<S>::value) return true;
+  constexpr int rows = std::is_same<S, SF32B>::value ? 3 : 6;
+  constexpr unsigned full = BX == 64 ? 5 : (BX == 128 ? 3 : 2);  // CTAs an SM
+  const unsigned sms = (unsigned)device_sm_count();
+  return a.yc < rows || 2 * grid < sms || grid >= full * sms;
+}
+
 template <int MODEL, class S, int BX, int NS>
 static cudaError_t launch_staged(const OpArgs& a, cudaStream_t s) {
   using L = TmaLayout<MODEL, S, BX, NS>;
@@ -131,6 +153,7 @@ static cudaError_t launch_staged(const OpArgs& a, cudaStream_t s) {
   k.yc = a.yc;
   k.err = a.err;
   const unsigned grid = tiles_1d((a.nx + BX - 1) / BX, a.ny, a.yc);
+  k.early = early_trigger<S, BX>(a, grid);
   return launch_pdl(step_tma_kernel<MODEL, S, BX, NS>, grid, BX + 32, L::BYTES, s, k);
 }
 

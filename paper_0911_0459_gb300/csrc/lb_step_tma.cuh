@@ -191,6 +191,7 @@ struct TmaArgs {
   MomPhys Q;  // the pair-form constants (storages that compute in deviations)
   Buf<S> src, dst;
   int yc;
+  int early;  // let the next step's CTAs in when this CTA's rows are on their way, not when it is done
   int* err;  // set to 1 when a wait gave up
 };
 
@@ -772,7 +773,7 @@ __global__ void __launch_bounds__(BX + 32, (tma_min_blocks_of<MODEL, S, BX, NS>(
     if (lane != 0) return;
     unsigned issued = 0;
     if (!produce_tile<MODEL, S, BX, NS>(R, a.G, a.src, xb, y0, y1, 0u, issued)) atomicExch(a.err, 1);
-    pdl_trigger();
+    if (a.early) pdl_trigger();
     drain_ring<MODEL, S, BX, NS>(R, issued);
     return;
   }

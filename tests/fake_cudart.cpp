@@ -31,6 +31,7 @@ struct Cost {
 };
 std::vector<Cost> costs;
 std::map<std::string, int> resident;
+std::map<std::string, unsigned> watched;  // byte of a kernel's first argument at which a word is logged
 std::map<uintptr_t, double> clocks;  // us, by stream
 uintptr_t handles = 0x1000;
 struct Launch {
@@ -106,6 +107,8 @@ void fake_resident(const char* kernel, int per_sm) {
   resident[kernel] = per_sm;
 }
 
+void fake_watch(const char* kernel, unsigned offset) { watched[kernel] = offset; }
+
 // ---- the library's side
 void** __cudaRegisterFatBinary(void*) { return (void**)handle(); }
 void __cudaRegisterFatBinaryEnd(void**) {}
@@ -142,8 +145,11 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void**, size_t sm
 cudaError_t cudaLaunchKernel(const void* f, dim3 g, dim3 b, void**, size_t smem, cudaStream_t s) {
   return launch(f, g, b, smem, s);
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
   FAIL(cudaLaunchKernelExC);
+  const std::string n = name_of(f);
+  for (const auto& w : watched)
+    if (n.find(w.first) != std::string::npos) note("word %d", *(const int*)((const char*)args[0] + w.second));
   return launch(f, c->gridDim, c->blockDim, c->dynamicSmemBytes, c->stream);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {

@@ -1,5 +1,9 @@
 """The step kernel behind the automatic choice, by lattice and tile, without a GPU (fake_cudart.cpp)."""
-from fake_cuda import run
+import json
+import os
+import subprocess
+
+from fake_cuda import ROOT, run
 
 
 def test_tall_bands_on_small_block_lattices_run_the_staged_kernel(tmp_path):
@@ -72,3 +76,44 @@ print(json.dumps(seen))
         if not strip:
             windows.add((nx, tx, ty, st))
     assert {(2304, 128, 4, 1), (2304, 64, 4, 2), (1024, 256, 2, 0)} <= windows
+
+
+def test_staged_launches_that_let_the_next_step_in_early(tmp_path):
+    """TmaArgs::early: off for long CTAs between half of one and five (64 columns), three (128), two
+    (256) on each of the 152 SMs: FP64 bands from six rows, FP32 blocks from three, FP16 blocks
+    from six; on for everything else."""
+    from paper_0911_0459_gb300 import build
+    kinds = [(m, s) for m, s in ((0, "SF64"), (1, "SF64"), (1, "SF32"), (0, "SF32"), (1, "SF16"), (1, "SF32B"), (1, "SF16B"))]
+    probe = tmp_path / "offsets.cu"
+    probe.write_text('#include <stddef.h>\n#include <stdio.h>\n#include "lb_step_tma.cuh"\nint main() {\n' + "".join(
+        f'  {{ using T = lbk::TmaArgs<{m}, lbk::{s}>; printf("%zu\\n", offsetof(T, early)); }}\n' for m, s in kinds) + "}\n")
+    subprocess.run([build.nvcc(), "-std=c++17", *build.ARCH, "-I", os.path.join(ROOT, "include"), "-I", build.CSRC, "-o",
+                    str(tmp_path / "offsets"), str(probe)], check=True, capture_output=True)
+    at = subprocess.run([str(tmp_path / "offsets")], capture_output=True, text=True, check=True).stdout.split()
+    watch = {f"step_tma_kernel<{m}, lbk::{s}, ": int(o) for (m, s), o in zip(kinds, at)}
+    seen = run(tmp_path, "for k, o in " + json.dumps(watch) + ".items(): fake.fake_watch(k.encode(), o)\n" + r'''
+seen = []
+for nx, ny in ((1024, 64), (1000, 200), (4096, 128)):
+    for model, st in ((W.LG, lb.STORAGE_F64), (W.BINARY, lb.STORAGE_F64), (W.BINARY, lb.STORAGE_F32), (W.LG, lb.STORAGE_F32),
+                      (W.BINARY, lb.STORAGE_F16DEV), (W.BINARY, lb.STORAGE_F32_BLOCKED), (W.BINARY, lb.STORAGE_F16_BLOCKED)):
+        h = lattice(nx, ny, model, st)
+        for v in (2, 3):
+            assert L.lb_set_kernel(h, v) == 0
+            for t in [(x, y) for x in (64, 128, 256) for y in (1, 2, 3, 5, 6, 12, 32)]:
+                assert L.lb_set_tile(h, *t) == 0
+                log()
+                assert L.lb_step(h, 1) == 0
+                lines = log()
+                (i, l), = [(i, l) for i, l in enumerate(lines) if l[0] == "launch"]
+                assert "step_tma_kernel" in l[5] and lines[i - 1][0] == "word"
+                seen.append([st, t, int(l[2]), int(lines[i - 1][1])])
+        L.lb_destroy(h)
+print(json.dumps(seen))
+''')
+    late = 0
+    for st, (tx, ty), grid, early in seen:
+        rows, full = {0: 6, 6: 3, 7: 6}.get(st), {64: 5, 128: 3, 256: 2}[tx]
+        expect = rows is None or ty < rows or not 76 <= grid < full * 152
+        assert early == expect, (st, tx, ty, grid)
+        late += not early
+    assert late > 30
