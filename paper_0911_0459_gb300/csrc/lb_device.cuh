@@ -518,6 +518,8 @@ struct Buf {
 // 5.11 us, 700 x 40 FP32 planes 3.61 -> 3.47 us, 16384 x 256 unchanged.  A CTA lets
 // its dependents in when its own rows are done (pdl_trigger): let in at the start
 // they took the slots of idle SMs unevenly (256 x 32 FP64: 11.6 instead of 8.6 us).
+// A CTA of the staged kernel does so when its last row is on its way, unless that has the
+// same effect (early_trigger).
 // The moment kernel keeps plain launches (1024 x 64: 4.79 us, 5.37 us with this).
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
